@@ -38,41 +38,31 @@ lattice_batch_kernel(const BatchLattice<C>* __restrict__ cases, const int* __res
                                    band_stamp_after(d.stamp, k + 1));
 }
 
-// The same over the particles of many cases, step k of a batch call.
-__global__ void __launch_bounds__(32 * STEP_WARPS, 1)
+// The same over the particles of many cases, step k of a batch call; `group`
+// (case, particle) items per CTA (see step_group).
+__global__ void __launch_bounds__(STEP_THREADS)
     particle_step_batch_kernel(const BatchParticles* __restrict__ cases, const int2* __restrict__ items, int nitems,
-                               int k) {
-  __shared__ int s_queue[STEP_WARPS][BAND_QUEUE];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int i0 = blockIdx.x * STEP_WARPS;
-  if (warp == 0 && lane < STEP_WARPS && i0 + lane < nitems) {
-    const int2 it = items[i0 + lane];
+                               int k, int group) {
+  __shared__ StepShared sh;
+  const int i0 = blockIdx.x * group;
+  step_group(min(group, nitems - i0), [&](int s) {
+    const int2 it = items[i0 + s];
     const BatchParticles& d = cases[it.x];
-    advance_one(d.c, d.P, it.y, d.err);
-  }
-  __syncthreads();
-  const int i = i0 + warp;
-  if (i >= nitems) return;  // the whole warp
-  const int2 it = items[i];
-  const BatchParticles& d = cases[it.x];
-  if (d.P.rb[it.y] != d.P.r[it.y]) return;
-  const int nl = 1 - (d.tl ^ (k & 1));
-  band_one<false>(d.c, d.P, d.TL[nl], d.err, it.y, band_stamp_after(d.stamp, k + 1), s_queue[warp], lane);
+    return StepRef{&d.c, &d.P, &d.TL[1 - (d.tl ^ (k & 1))], d.err, it.y, band_stamp_after(d.stamp, k + 1)};
+  }, sh);
 }
-// The ellipses' band pass of step k (of step *kdev when kdev is given).
-__global__ void __launch_bounds__(32 * BAND_WARPS)
-    particle_band_ellipse_batch_kernel(const BatchParticles* __restrict__ cases, const int2* __restrict__ items,
-                                       int nitems, int k, const int* __restrict__ kdev) {
-  __shared__ int s_queue[BAND_WARPS][BAND_QUEUE];
+// The ellipses' band tables of step k (of step *kdev when kdev is given).
+__global__ void __launch_bounds__(32 * ELL_WARPS)
+    particle_ellipse_batch_kernel(const BatchParticles* __restrict__ cases, const int2* __restrict__ items, int blocks,
+                                  int k, const int* __restrict__ kdev) {
+  __shared__ int s_queue[ELL_WARPS][32];
   if (kdev) k = *kdev;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int i = blockIdx.x * BAND_WARPS + warp;
-  if (i >= nitems) return;  // the whole warp
+  const int i = blockIdx.x / blocks, by = (blockIdx.x - i * blocks) * ELL_WARPS + warp;
   const int2 it = items[i];
   const BatchParticles& d = cases[it.x];
-  if (d.P.rb[it.y] == d.P.r[it.y]) return;
-  const int nl = 1 - (d.tl ^ (k & 1));
-  band_one<true>(d.c, d.P, d.TL[nl], d.err, it.y, band_stamp_after(d.stamp, k + 1), s_queue[warp], lane);
+  if (by >= 2 * d.c.band_off + 1) return;  // the whole warp
+  ellipse_row(d.c, d.P, it.y, band_stamp_after(d.stamp, k + 1), by, lane, s_queue[warp]);
 }
 
 template <class S, class C>
@@ -96,22 +86,22 @@ cudaError_t launch_lattice_batch_f64(const BatchLattice<double>* cases, const in
   return launch_batch<double, double>(cases, tile_case, ntiles, k, held, st);
 }
 
-cudaError_t launch_particle_step_batch(const BatchParticles* cases, const int2* items, int nitems, int k,
-                                       bool any_ellipse, cudaStream_t st) {
-  if (nitems == 0) return cudaSuccess;
-  particle_step_batch_kernel<<<(unsigned)((nitems + STEP_WARPS - 1) / STEP_WARPS), 32 * STEP_WARPS, 0, st>>>(
-      cases, items, nitems, k);
-  if (any_ellipse)
-    particle_band_ellipse_batch_kernel<<<(unsigned)((nitems + BAND_WARPS - 1) / BAND_WARPS), 32 * BAND_WARPS, 0, st>>>(
-        cases, items, nitems, k, nullptr);
+cudaError_t launch_ellipse_batch(const BatchParticles* cases, const BatchEllipses& ell, int k, const int* kdev,
+                                 cudaStream_t st) {
+  if (ell.n == 0) return cudaSuccess;
+  const int blocks = (ell.rows + ELL_WARPS - 1) / ELL_WARPS;
+  particle_ellipse_batch_kernel<<<(unsigned)(blocks * ell.n), 32 * ELL_WARPS, 0, st>>>(cases, ell.items, blocks, k,
+                                                                                      kdev);
   return cudaGetLastError();
 }
-cudaError_t launch_particle_band_ellipse_batch(const BatchParticles* cases, const int2* items, int nitems, int k,
-                                               const int* kdev, cudaStream_t st) {
+cudaError_t launch_particle_step_batch(const BatchParticles* cases, const int2* items, int nitems, int k,
+                                       const BatchEllipses& ell, cudaStream_t st) {
   if (nitems == 0) return cudaSuccess;
-  particle_band_ellipse_batch_kernel<<<(unsigned)((nitems + BAND_WARPS - 1) / BAND_WARPS), 32 * BAND_WARPS, 0, st>>>(
-      cases, items, nitems, k, kdev);
-  return cudaGetLastError();
+  const int group = step_group_size(nitems);
+  particle_step_batch_kernel<<<(unsigned)((nitems + group - 1) / group), STEP_THREADS, 0, st>>>(cases, items, nitems, k,
+                                                                                               group);
+  const cudaError_t e = cudaGetLastError();
+  return e != cudaSuccess ? e : launch_ellipse_batch(cases, ell, k, nullptr, st);
 }
 
 // ---- the persistent form ------------------------------------------------------
@@ -158,13 +148,17 @@ __device__ __forceinline__ void persistent_particle(const PersistentBatch<C>& A,
   if (lane == 0) {
     const LatticeConst<C>& K = A.cases[it.x].K;
     ok = wait_count(A.done + it.x, K.ntx * K.nty + (it.x == A.stuck_case ? 1 : 0), A.wait_ns);
-    if (ok) advance_one(pd.c, pd.P, it.y, pd.err);
-    else atomicOr(pd.err, ERR_TIMEOUT);
+    if (!ok) atomicOr(pd.err, ERR_TIMEOUT);
   }
   ok = __shfl_sync(0xffffffffu, ok, 0);
-  if (ok && pd.P.rb[it.y] == pd.P.r[it.y])
-    band_one<false>(pd.c, pd.P, pd.TL[1 - (pd.tl ^ (kn & 1))], pd.err, it.y, band_stamp_after(pd.stamp, kn + 1), queue,
-                    lane);
+  if (!ok) return;  // the whole warp
+  __syncwarp();     // what lane 0 waited for is visible to every lane
+  const UpdateLane u = update_position(pd.c, pd.P, it.y, lane, lane < 4, pd.err);
+  RasterRec rq;
+  record_constants(pd.P, it.y, u.R, u.Rb, rq);
+  update_velocity(pd.c, pd.P, it.y, lane, lane < 4, u, rq, pd.err);
+  __syncwarp();  // the record and tile range are visible to every lane
+  band_one(pd.c, pd.P, pd.TL[1 - (pd.tl ^ (kn & 1))], pd.err, it.y, band_stamp_after(pd.stamp, kn + 1), queue, lane);
 }
 
 // Tiles per work chunk of the persistent launch: a CTA takes the next chunk

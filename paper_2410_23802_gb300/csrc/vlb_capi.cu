@@ -59,6 +59,8 @@ struct vlb_handle {
   int tl = 0;  // list buffer of the current level
   void* pbase = nullptr;
   size_t pbytes = 0;  // bytes of the particle block at pbase
+  int* ell = nullptr;  // the particles that are ellipses, on the device (null: none)
+  int nell = 0;
   // device error word and its pinned host copy (refreshed in stream order)
   unsigned* err_host = nullptr;
   bool err_host_external = false;  // the served mode's arena owns it
@@ -219,6 +221,7 @@ static void free_all(vlb_handle* h) {
     dev_free(h, h->TL[b].count);
     dev_free(h, h->TL[b].ids);
   }
+  dev_free(h, h->ell);
   dev_free(h, h->P.mes);
   dev_free(h, h->P.band);
   dev_free(h, h->audit_scratch);
@@ -594,6 +597,20 @@ static vlb_status upload_particles(vlb_handle* h, int first, int count) {
   return VLB_OK;
 }
 
+// The list of the ellipses (after the host's axes are known).
+static vlb_status upload_ellipses(vlb_handle* h) {
+  std::vector<int> ids;
+  for (int k = 0; k < h->np; ++k)
+    if (h->hrb[k] != h->hr[k]) ids.push_back(k);
+  h->nell = (int)ids.size();
+  if (ids.empty()) return VLB_OK;
+  // (room for every particle: a loaded state may hold other axes)
+  if (!h->ell) CK(h, dev_alloc(h, reinterpret_cast<void**>(&h->ell), (size_t)std::max(h->cap, 1) * sizeof(int)));
+  CK(h, cudaMemcpyAsync(h->ell, ids.data(), ids.size() * sizeof(int), cudaMemcpyHostToDevice, h->stream));
+  CK(h, cudaStreamSynchronize(h->stream));  // the list on the host ends here
+  return VLB_OK;
+}
+
 static vlb_status initialize(vlb_handle* h) {
   const vlb_params& p = h->p;
   const int n = h->np;
@@ -629,8 +646,6 @@ static vlb_status initialize(vlb_handle* h) {
   int any_held = 0;
   for (int v : h->hfix) any_held |= v;
   h->K32.any_held = h->K64.any_held = any_held;
-  c.any_ellipse = 0;
-  for (size_t k = 0; k < h->hr.size(); ++k) c.any_ellipse |= h->hrb[k] != h->hr[k];
   c.rho_ratio = p.rho_ratio; c.gx = p.gravity[0]; c.gy = p.gravity[1];
   c.zeta = p.contact_range; c.eps_p = p.contact_eps_p; c.eps_w = p.contact_eps_w;
   c.contact_scale = std::fabs(p.rho_ratio - 1.0) * std::hypot(p.gravity[0], p.gravity[1]) * M_PI;
@@ -642,7 +657,8 @@ static vlb_status initialize(vlb_handle* h) {
   CK(h, launch_particle_range(c, h->P, h->err_dev, h->stream));
   h->tl = 0;
   next_band_stamp(h);
-  CK(h, launch_particle_band(c, h->P, h->TL[0], h->err_dev, h->stream));
+  if (vlb_status st = upload_ellipses(h); st != VLB_OK) return st;
+  CK(h, launch_particle_band(c, h->P, h->TL[0], h->ell, h->nell, h->err_dev, h->stream));
   h->cur = 0;
   vlb_status s = launch_lattice(h, MODE_INIT, 0, 0, 0);
   if (s != VLB_OK) return s;
@@ -657,7 +673,7 @@ static vlb_status step_once(vlb_handle* h) {
   vlb_status s;
   const int nl = 1 - h->tl;
   next_band_stamp(h);
-  CK(h, launch_particle_step(h->PC, h->P, h->TL[nl], h->err_dev, h->stream));
+  CK(h, launch_particle_step(h->PC, h->P, h->TL[nl], h->ell, h->nell, h->err_dev, h->stream));
   const bool rec = h->prof && h->ev_used + 2 <= h->ev_cap;
   if (rec) CK(h, cudaEventRecord(h->ev[h->ev_used], h->stream));
   if ((s = launch_lattice(h, MODE_STEP, h->cur, 1 - h->cur, nl)) != VLB_OK) return s;
@@ -869,7 +885,8 @@ static vlb_status step_batch_impl(vlb_handle* const* hs, int32_t n, int32_t nste
   const int h0dev = hs[0]->device;
   const bool persistent = g_batch_form.load() == 1;
   std::vector<BatchGroup> groups;
-  std::vector<int2> items;
+  std::vector<int2> items, eitems;
+  int erows = 0;
   for (int i = 0; i < n; ++i) {
     vlb_handle* h = hs[i];
     const bool f64 = h->p.precision == VLB_FP64;
@@ -887,10 +904,17 @@ static vlb_status step_batch_impl(vlb_handle* const* hs, int32_t n, int32_t nste
     }
     g->handles.push_back(i);
     for (int k = 0; k < h->np; ++k) items.push_back(make_int2(i, k));
+    if (h->nell > 0) {
+      for (int k = 0; k < h->np; ++k)
+        if (h->hrb[k] != h->hr[k]) eitems.push_back(make_int2(i, k));
+      erows = std::max(erows, 2 * h->PC.band_off + 1);
+    }
   }
   size_t bytes = align16(sizeof(BatchParticles) * n);
   const size_t items_off = bytes;
   bytes = align16(bytes + sizeof(int2) * items.size());
+  const size_t eitems_off = bytes;
+  bytes = align16(bytes + sizeof(int2) * eitems.size());
   for (auto& g : groups) {
     long long nt = 0;
     for (int i : g.handles) nt += (long long)hs[i]->ntx * hs[i]->nty;
@@ -948,6 +972,7 @@ static vlb_status step_batch_impl(vlb_handle* const* hs, int32_t n, int32_t nste
     bp[i] = d;
   }
   if (!items.empty()) std::memcpy(hostp + items_off, items.data(), sizeof(int2) * items.size());
+  if (!eitems.empty()) std::memcpy(hostp + eitems_off, eitems.data(), sizeof(int2) * eitems.size());
   for (auto& g : groups) {
     int* table = reinterpret_cast<int*>(hostp + g.table_off);
     int tile0 = 0;
@@ -981,11 +1006,10 @@ static vlb_status step_batch_impl(vlb_handle* const* hs, int32_t n, int32_t nste
   const auto* d_part = reinterpret_cast<const BatchParticles*>(dev);
   const auto* d_items = reinterpret_cast<const int2*>(dev + items_off);
   const int nitems = (int)items.size();
-  bool any_ellipse = false;
-  for (int i = 0; i < n; ++i) any_ellipse |= hs[i]->PC.any_ellipse != 0;
+  const BatchEllipses ell{reinterpret_cast<const int2*>(dev + eitems_off), (int)eitems.size(), erows};
   if (!persistent) {
     for (int k = 0; k < nsteps && e == cudaSuccess; ++k) {
-      e = launch_particle_step_batch(d_part, d_items, nitems, k, any_ellipse, bs);
+      e = launch_particle_step_batch(d_part, d_items, nitems, k, ell, bs);
       for (auto& g : groups) {
         if (e != cudaSuccess) break;
         const int* table = reinterpret_cast<const int*>(dev + g.table_off);
@@ -1017,12 +1041,11 @@ static vlb_status step_batch_impl(vlb_handle* const* hs, int32_t n, int32_t nste
         }
         if (el != cudaSuccess) return el;
       }
-      if (with_particles && any_ellipse)
-        return launch_particle_band_ellipse_batch(d_part, d_items, nitems, 0,
-                                                  &reinterpret_cast<const BatchCtl*>(dev + groups[0].ctl_off)->k, bs);
+      if (with_particles)
+        return launch_ellipse_batch(d_part, ell, 0, &reinterpret_cast<const BatchCtl*>(dev + groups[0].ctl_off)->k, bs);
       return cudaSuccess;
     };
-    e = launch_particle_step_batch(d_part, d_items, nitems, 0, any_ellipse, bs);
+    e = launch_particle_step_batch(d_part, d_items, nitems, 0, ell, bs);
     // the steps' launches are the same every step (the step index lives on
     // the device): up to kGraphSteps of them are captured into one CUDA graph,
     // replayed as often as it fits, and the rest launched plainly
@@ -1490,8 +1513,7 @@ vlb_status vlb_load_state(vlb_handle* h, const void* buf, uint64_t bytes) {
   int any_held = 0;
   for (int v : h->hfix) any_held |= v;
   h->K32.any_held = h->K64.any_held = any_held;
-  h->PC.any_ellipse = 0;
-  for (int k = 0; k < h->np; ++k) h->PC.any_ellipse |= h->hrb[k] != h->hr[k];
+  if ((s = upload_ellipses(h)) != VLB_OK) return s;
   h->cur = I.cur;
   h->tl = I.tl;
   h->step = I.step;
@@ -1529,7 +1551,7 @@ vlb_status vlb_profile_end(vlb_handle* h, double* lattice_ms, int32_t* lattice_l
   if (lattice_ms) *lattice_ms = tot;
   if (lattice_launches) *lattice_launches = h->ev_used / 2;
   // particle_step (and the ellipses' band pass) and the lattice kernel
-  if (launches_per_step) *launches_per_step = h->np > 0 ? (h->PC.any_ellipse ? 3 : 2) : 1;
+  if (launches_per_step) *launches_per_step = h->np > 0 ? (h->nell > 0 ? 3 : 2) : 1;
   h->prof = false;
   h->ev_used = 0;
   return VLB_OK;

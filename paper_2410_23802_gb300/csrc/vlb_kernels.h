@@ -9,7 +9,6 @@ namespace vlb {
 struct ParticleConst {
   int np, nx, ny, per_x, per_y, ntx, nty;
   int outflow[4];    // open sides (no wall contact there)
-  int any_ellipse;   // some particle is an ellipse (its band pass runs in a kernel of its own)
   int band_off;      // half-width of the band tables (cells)
   int band_stamp;    // level stamp written into the band tables
   double rho_ratio, gx, gy;
@@ -57,18 +56,23 @@ cudaError_t launch_raster_dump_f64(const LatticeConst<double>& K, const Particle
                                    const TileLists& TL, unsigned char* count, int* owner,
                                    unsigned char* flag, double* fsp, unsigned* err, cudaStream_t st);
 
-// Particle step pieces.
+// Particle step pieces (ell[nell]: the particles that are ellipses, on the device).
 cudaError_t launch_particle_range(const ParticleConst& c, const ParticleArrays& P, unsigned* err,
                                   cudaStream_t st);
-cudaError_t launch_particle_band(const ParticleConst& c, const ParticleArrays& P, const TileLists& TL, unsigned* err,
-                                 cudaStream_t st);
+cudaError_t launch_particle_band(const ParticleConst& c, const ParticleArrays& P, const TileLists& TL, const int* ell,
+                                 int nell, unsigned* err, cudaStream_t st);
 
-// Advance and band pass of every particle in one launch (list buffer TL, the
-// stamp of ParticleConst).
-cudaError_t launch_particle_step(const ParticleConst& c, const ParticleArrays& P, const TileLists& TL, unsigned* err,
-                                 cudaStream_t st);
+// Update, lists and band tables of every particle (list buffer TL, the stamp
+// of ParticleConst).
+cudaError_t launch_particle_step(const ParticleConst& c, const ParticleArrays& P, const TileLists& TL, const int* ell,
+                                 int nell, unsigned* err, cudaStream_t st);
+// The (case, ellipse) pairs of a batch, on the device, and the most rows of their boxes.
+struct BatchEllipses {
+  const int2* items;
+  int n, rows;
+};
 cudaError_t launch_particle_step_batch(const BatchParticles* cases, const int2* items, int nitems, int k,
-                                       bool any_ellipse, cudaStream_t st);
+                                       const BatchEllipses& ell, cudaStream_t st);
 
 // Batched step k: lattice tiles map to their case through tile_case.
 // `held`: the held-temperature path (every case of the launch shares
@@ -111,10 +115,10 @@ int persistent_grid(int device, bool f64, int storage, bool held);
 cudaError_t launch_lattice_persistent_f32(const PersistentBatch<float>& A, int grid, int storage, bool held,
                                           cudaStream_t st);
 cudaError_t launch_lattice_persistent_f64(const PersistentBatch<double>& A, int grid, bool held, cudaStream_t st);
-// The band pass of the batch's ellipses for step k, or for step *kdev when
+// The band tables of the batch's ellipses for step k, or for step *kdev when
 // kdev is given (the level a persistent launch has just advanced to).
-cudaError_t launch_particle_band_ellipse_batch(const BatchParticles* cases, const int2* items, int nitems, int k,
-                                               const int* kdev, cudaStream_t st);
+cudaError_t launch_ellipse_batch(const BatchParticles* cases, const BatchEllipses& ell, int k, const int* kdev,
+                                 cudaStream_t st);
 
 // FP64 audits: out[0] = sum f, out[1] = sum eps, out[2] = sum g (block partials
 // in scratch[3 * nblocks], summed in block order).

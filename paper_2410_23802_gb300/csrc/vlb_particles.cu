@@ -11,36 +11,37 @@ __global__ void particle_range_kernel(const ParticleConst c, const ParticleArray
   write_record(P, p, P.x[p], P.y[p], P.r[p], P.rb[p], P.ux[p], P.uy[p], P.om[p], float(P.lam_s[p]), float(P.T0[p]));
 }
 
-// The band pass of every disk (ELL false) or of every ellipse (ELL true),
-// one warp per particle; the particles of the other kind are left alone.
-template <bool ELL>
+// Lists of every particle and band tables of the disks at the initial state,
+// one warp per particle.
 __global__ void __launch_bounds__(32 * BAND_WARPS) particle_band_kernel(const ParticleConst c, const ParticleArrays P,
                                                                         const TileLists TL, unsigned* err) {
   __shared__ int s_queue[BAND_WARPS][BAND_QUEUE];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int p = blockIdx.x * BAND_WARPS + warp;
-  if (p >= c.np || ((P.rb[p] != P.r[p]) != ELL)) return;  // the whole warp
-  band_one<ELL>(c, P, TL, err, p, c.band_stamp, s_queue[warp], lane);
+  if (p >= c.np) return;  // the whole warp
+  band_one(c, P, TL, err, p, c.band_stamp, s_queue[warp], lane);
 }
 
-// One particle step (advance, then lists and band table) in one launch: the
-// two depend on the particle alone.  A CTA of STEP_WARPS warps takes
-// STEP_WARPS particles: warp 0 advances them, one lane each (so the FP64
-// instructions stay shared by many particles and the advance is spread over
-// the SMs), then each warp runs the band pass of one of them; the barrier
-// between makes the new records visible.  Ellipses get their band pass from
-// particle_band_kernel<true> after this kernel.
-
-__global__ void __launch_bounds__(32 * STEP_WARPS, 1) particle_step_kernel(const ParticleConst c, const ParticleArrays P,
-                                                                        const TileLists TL, unsigned* err) {
-  __shared__ int s_queue[STEP_WARPS][BAND_QUEUE];
+// Band tables of the ellipses ell[0 .. n - 1], one warp per row.
+__global__ void __launch_bounds__(32 * ELL_WARPS)
+    particle_ellipse_kernel(const ParticleConst c, const ParticleArrays P, const int* __restrict__ ell, int blocks) {
+  __shared__ int s_queue[ELL_WARPS][32];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int p0 = blockIdx.x * STEP_WARPS;
-  if (warp == 0 && lane < STEP_WARPS && p0 + lane < c.np) advance_one(c, P, p0 + lane, err);
-  __syncthreads();
-  const int p = p0 + warp;
-  if (p >= c.np || P.rb[p] != P.r[p]) return;  // the whole warp
-  band_one<false>(c, P, TL, err, p, c.band_stamp, s_queue[warp], lane);
+  const int i = blockIdx.x / blocks, by = (blockIdx.x - i * blocks) * ELL_WARPS + warp;
+  if (by >= 2 * c.band_off + 1) return;  // the whole warp
+  ellipse_row(c, P, ell[i], c.band_stamp, by, lane, s_queue[warp]);
+}
+
+// One particle step (update, then lists and band tables) in one launch: the
+// two depend on the particle alone (see step_group).  `group` particles per
+// CTA.  Ellipses get their band tables from particle_ellipse_kernel after it.
+__global__ void __launch_bounds__(STEP_THREADS) particle_step_kernel(const __grid_constant__ ParticleConst c,
+                                                                     const __grid_constant__ ParticleArrays P,
+                                                                     const __grid_constant__ TileLists TL,
+                                                                     unsigned* err, int group) {
+  __shared__ StepShared sh;
+  const int p0 = blockIdx.x * group;
+  step_group(min(group, c.np - p0), [&](int s) { return StepRef{&c, &P, &TL, err, p0 + s, c.band_stamp}; }, sh);
 }
 
 static inline dim3 pgrid(int n) { return dim3((unsigned)((n + 127) / 128)); }
@@ -51,21 +52,26 @@ cudaError_t launch_particle_range(const ParticleConst& c, const ParticleArrays& 
   particle_range_kernel<<<pgrid(c.np), 128, 0, st>>>(c, P, err);
   return cudaGetLastError();
 }
-cudaError_t launch_particle_band(const ParticleConst& c, const ParticleArrays& P, const TileLists& TL, unsigned* err,
-                                 cudaStream_t st) {
-  if (c.np == 0) return cudaSuccess;
-  const unsigned grid = (unsigned)((c.np + BAND_WARPS - 1) / BAND_WARPS);
-  particle_band_kernel<false><<<grid, 32 * BAND_WARPS, 0, st>>>(c, P, TL, err);
-  if (c.any_ellipse) particle_band_kernel<true><<<grid, 32 * BAND_WARPS, 0, st>>>(c, P, TL, err);
+static cudaError_t launch_ellipses(const ParticleConst& c, const ParticleArrays& P, const int* ell, int nell,
+                                   cudaStream_t st) {
+  if (nell > 0) {
+    const int blocks = (2 * c.band_off + ELL_WARPS) / ELL_WARPS;  // rows 0 .. 2 band_off
+    particle_ellipse_kernel<<<(unsigned)(blocks * nell), 32 * ELL_WARPS, 0, st>>>(c, P, ell, blocks);
+  }
   return cudaGetLastError();
 }
-cudaError_t launch_particle_step(const ParticleConst& c, const ParticleArrays& P, const TileLists& TL, unsigned* err,
-                                 cudaStream_t st) {
+cudaError_t launch_particle_band(const ParticleConst& c, const ParticleArrays& P, const TileLists& TL, const int* ell,
+                                 int nell, unsigned* err, cudaStream_t st) {
   if (c.np == 0) return cudaSuccess;
-  particle_step_kernel<<<(unsigned)((c.np + STEP_WARPS - 1) / STEP_WARPS), 32 * STEP_WARPS, 0, st>>>(c, P, TL, err);
-  if (c.any_ellipse)
-    particle_band_kernel<true><<<(unsigned)((c.np + BAND_WARPS - 1) / BAND_WARPS), 32 * BAND_WARPS, 0, st>>>(c, P, TL,
-                                                                                                          err);
-  return cudaGetLastError();
+  const unsigned grid = (unsigned)((c.np + BAND_WARPS - 1) / BAND_WARPS);
+  particle_band_kernel<<<grid, 32 * BAND_WARPS, 0, st>>>(c, P, TL, err);
+  return launch_ellipses(c, P, ell, nell, st);
+}
+cudaError_t launch_particle_step(const ParticleConst& c, const ParticleArrays& P, const TileLists& TL, const int* ell,
+                                 int nell, unsigned* err, cudaStream_t st) {
+  if (c.np == 0) return cudaSuccess;
+  const int group = step_group_size(c.np);
+  particle_step_kernel<<<(unsigned)((c.np + group - 1) / group), STEP_THREADS, 0, st>>>(c, P, TL, err, group);
+  return launch_ellipses(c, P, ell, nell, st);
 }
 }  // namespace vlb

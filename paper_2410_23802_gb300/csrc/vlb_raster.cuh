@@ -50,6 +50,21 @@ __host__ __device__ __forceinline__ double add_rn(double a, double b) {
 #endif
 }
 
+__host__ __device__ __forceinline__ float fma_rn(float a, float b, float c) {
+#ifdef __CUDA_ARCH__
+  return __fmaf_rn(a, b, c);
+#else
+  return fmaf(a, b, c);
+#endif
+}
+__host__ __device__ __forceinline__ double fma_rn(double a, double b, double c) {
+#ifdef __CUDA_ARCH__
+  return __fma_rn(a, b, c);
+#else
+  return fma(a, b, c);
+#endif
+}
+
 enum : int { CELL_FLUID = 0, CELL_INTERFACE = 1, CELL_SOLID = 2 };
 
 // An ellipse as the FP64 lattice kernel sees it (the FP32 kernel reads
@@ -78,46 +93,73 @@ struct PartTile : EllPart<C> {
   int rx, ry;             // first tile of the particle's range
 };
 
+// Class of the cell whose lower-left corner lies at (cx0, cy0) from the disk's
+// centre (2^-20 grid).  I: long long, or int where every |cx0| + 2^20 fits 31
+// bits (each product is then one 32 x 32 -> 64 bit multiply).
+template <class I>
+__host__ __device__ __forceinline__ int cell_class_at(I cx0, I cy0, long long rq2) {
+  const I Q = I(1) << QBITS;
+  const I cx1 = cx0 + Q, cy1 = cy0 + Q;
+  const I ax0 = cx0 < 0 ? -cx0 : cx0, ax1 = cx1 < 0 ? -cx1 : cx1;
+  const I ay0 = cy0 < 0 ? -cy0 : cy0, ay1 = cy1 < 0 ? -cy1 : cy1;
+  const I fx = ax0 > ax1 ? ax0 : ax1, fy = ay0 > ay1 ? ay0 : ay1;  // farthest corner
+  if ((long long)fx * fx + (long long)fy * fy <= rq2) return CELL_SOLID;
+  const I nx = (cx0 <= 0 && cx1 >= 0) ? 0 : (ax0 < ax1 ? ax0 : ax1);  // nearest point
+  const I ny = (cy0 <= 0 && cy1 >= 0) ? 0 : (ay0 < ay1 ? ay0 : ay1);
+  if ((long long)nx * nx + (long long)ny * ny >= rq2) return CELL_FLUID;
+  return CELL_INTERFACE;
+}
 // Integer classification of cell (il, jl) of the tile against one disk.
 template <class C>
 __host__ __device__ __forceinline__ int cell_class_exact(int il, int jl, const PartTile<C>& p) {
   const long long Q = 1ll << QBITS;
-  const long long cx0 = (long long)il * Q - p.xq, cx1 = cx0 + Q;
-  const long long cy0 = (long long)jl * Q - p.yq, cy1 = cy0 + Q;
-  const long long fx = cx0 * cx0 > cx1 * cx1 ? cx0 * cx0 : cx1 * cx1;
-  const long long fy = cy0 * cy0 > cy1 * cy1 ? cy0 * cy0 : cy1 * cy1;
-  if (fx + fy <= p.rq2) return CELL_SOLID;
-  const long long ax0 = cx0 < 0 ? -cx0 : cx0, ax1 = cx1 < 0 ? -cx1 : cx1;
-  const long long ay0 = cy0 < 0 ? -cy0 : cy0, ay1 = cy1 < 0 ? -cy1 : cy1;
-  const long long nx = (cx0 <= 0 && cx1 >= 0) ? 0 : (ax0 < ax1 ? ax0 : ax1);
-  const long long ny = (cy0 <= 0 && cy1 >= 0) ? 0 : (ay0 < ay1 ? ay0 : ay1);
-  if (nx * nx + ny * ny >= p.rq2) return CELL_FLUID;
-  return CELL_INTERFACE;
+  return cell_class_at((long long)il * Q - p.xq, (long long)jl * Q - p.yq, p.rq2);
 }
 
-// Area of the circular segment cut off by a chord of length L (L <= 2R):
-// R^2 (asin z - z sqrt(1 - z^2)), z = L / (2R).
-__host__ __device__ __forceinline__ double segment_area(double L, double R) {
-  const double z = L / (2.0 * R);
-  return R * R * (asin(z) - z * sqrt(fmax(1.0 - z * z, 0.0)));
-}
-__host__ __device__ __forceinline__ float segment_area(float L, float R) {
-  const float z = L / (2.0f * R);
-  if (z < 0.25f) {
-    // Taylor series of asin z - z sqrt(1 - z^2):
-    // 2/3 z^3 + 1/5 z^5 + 3/28 z^7 + 5/72 z^9 + 35/704 z^11 + O(z^13)
-    const float z2 = z * z;
-    float s = 35.0f / 704.0f;
-    s = s * z2 + 5.0f / 72.0f;
-    s = s * z2 + 3.0f / 28.0f;
-    s = s * z2 + 0.2f;
-    s = s * z2 + 2.0f / 3.0f;
-    return R * R * s * z2 * z;
+// Area of the circular segment on a chord of squared length L2 (<= 4 R^2),
+// with i2R = 1 / (2R): R^2 (asin z - z sqrt(1 - z^2)), z = L / (2R).  Its
+// Taylor series is R^2 z^3 sum_k 2 b_k / (2k + 3) z^2k with b_k = C(2k, k) / 4^k
+// (the derivative is 2 z^2 / sqrt(1 - z^2)); for z below the given bound it is
+// cut where its terms pass the type's precision, and needs one square root
+// instead of three library calls and a division.
+__host__ __device__ __forceinline__ double segment_area(double L2, double R, double i2R) {
+  const double z2 = mul_rn(mul_rn(L2, i2R), i2R);
+  const double L = vsqrt(L2);
+  if (z2 < 1.0 / 64.0) {
+    double s = 12155.0 / 688128.0;
+    s = fma_rn(s, z2, 6435.0 / 311296.0);
+    s = fma_rn(s, z2, 429.0 / 17408.0);
+    s = fma_rn(s, z2, 77.0 / 2560.0);
+    s = fma_rn(s, z2, 63.0 / 1664.0);
+    s = fma_rn(s, z2, 35.0 / 704.0);
+    s = fma_rn(s, z2, 5.0 / 72.0);
+    s = fma_rn(s, z2, 3.0 / 28.0);
+    s = fma_rn(s, z2, 0.2);
+    s = fma_rn(s, z2, 2.0 / 3.0);
+    return mul_rn(mul_rn(mul_rn(L, L2), mul_rn(0.25, i2R)), s);
   }
-  return R * R * (asinf(z) - z * sqrtf(fmaxf(1.0f - z * z, 0.0f)));
+  double z = mul_rn(L, i2R);
+  z = z < 1.0 ? z : 1.0;
+  return mul_rn(mul_rn(R, R), add_rn(asin(z), -mul_rn(z, vsqrt(fma_rn(-z, z, 1.0)))));
+}
+__host__ __device__ __forceinline__ float segment_area(float L2, float R, float i2R) {
+  const float z2 = mul_rn(mul_rn(L2, i2R), i2R);
+  const float L = vsqrt(L2);
+  if (z2 < 0.0625f) {
+    float s = 35.0f / 704.0f;
+    s = fma_rn(s, z2, 5.0f / 72.0f);
+    s = fma_rn(s, z2, 3.0f / 28.0f);
+    s = fma_rn(s, z2, 0.2f);
+    s = fma_rn(s, z2, 2.0f / 3.0f);
+    return mul_rn(mul_rn(mul_rn(L, L2), mul_rn(0.25f, i2R)), s);
+  }
+  float z = mul_rn(L, i2R);
+  z = z < 1.0f ? z : 1.0f;
+  return mul_rn(mul_rn(R, R), add_rn(asinf(z), -mul_rn(z, vsqrt(fma_rn(-z, z, 1.0f)))));
 }
 
-// Exact area of disk((cx, cy), R) ∩ [0,1]^2 (cell-local coordinates), R >= 1.
+// Exact area of disk((cx, cy), R) ∩ [0,1]^2 (cell-local coordinates), R >= 1,
+// i2R = 1 / (2R).
 //
 // Walking the square's boundary counter-clockwise, each edge meets the closed
 // disk in one interval (possibly empty), found from that edge's own line.  The
@@ -127,56 +169,79 @@ __host__ __device__ __forceinline__ float segment_area(float L, float R) {
 // on its chord.  No entry/exit decision is taken: when rounding puts a circle
 // point on one or the other side of a corner, the link's chord is just tiny
 // and so is its segment.
+//
+// The four intervals are computed without branches (four independent square
+// roots in flight), the walk keeps the links' squared chords, and the segments
+// come last: a cell has one arc as a rule, so a warp evaluates one or two
+// segments where evaluating each link at its place in the walk cost it four.
+// Every operation is rounded on its own, so that the kernels that compute a
+// cell's area agree to the last bit however each was compiled.
 template <class C>
-__host__ __device__ __forceinline__ C disk_unit_cell_area(C cx, C cy, C R) {
-  // The polygon's points are visited in walking order (a_0, b_0, a_1, b_1, ...)
-  // and its shoelace terms and link segments summed on the fly, in that order,
-  // so no point list is kept.
-  C x0 = C(0), y0 = C(0);  // first point (a_0)
-  C xp = C(0), yp = C(0);  // last point so far
-  bool any = false;
-  C twice = C(0), seg = C(0);
+__host__ __device__ __forceinline__ C disk_unit_cell_area(C cx, C cy, C R, C i2R) {
+  // edge 0: y = 0, x 0 -> 1; edge 1: x = 1, y 0 -> 1; edge 2: y = 1, x 1 -> 0;
+  // edge 3: x = 0, y 1 -> 0
+  C lo[4], hi[4];
+  bool on[4];
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
-    // edge 0: y = 0, x 0 -> 1; edge 1: x = 1, y 0 -> 1; edge 2: y = 1, x 1 -> 0;
-    // edge 3: x = 0, y 1 -> 0
     const bool horiz = (k == 0 || k == 2);
-    const C fixed = (k == 1 || k == 2) ? C(1) : C(0);
-    const C d = fixed - (horiz ? cy : cx);
+    const C d = add_rn((k == 1 || k == 2) ? C(1) : C(0), -(horiz ? cy : cx));
     const C ad = d < C(0) ? -d : d;
-    if (ad >= R) continue;
-    const C s = vsqrt((R - ad) * (R + ad));
+    const bool meets = ad < R;
+    const C h = mul_rn(add_rn(R, -ad), add_rn(R, ad));
+    const C s = vsqrt(meets ? h : C(1));
     const C c_run = horiz ? cx : cy;
-    C lo = c_run - s, hi = c_run + s;
-    lo = lo < C(0) ? C(0) : lo;
-    hi = hi > C(1) ? C(1) : hi;
-    if (!(hi > lo)) continue;
-    const bool up = (k == 0 || k == 1);
-    const C a = up ? lo : hi, b = up ? hi : lo;  // start and end in walking order
+    lo[k] = add_rn(c_run, -s);
+    hi[k] = add_rn(c_run, s);
+    lo[k] = lo[k] < C(0) ? C(0) : lo[k];
+    hi[k] = hi[k] > C(1) ? C(1) : hi[k];
+    on[k] = meets && hi[k] > lo[k];
+  }
+  // the walk: interval ends (ax, ay) -> (bx, by) in order, links between them
+  C x0 = C(0), y0 = C(0), xp = C(0), yp = C(0);
+  C twice = C(0), l2[4];
+  bool any = false;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const bool horiz = (k == 0 || k == 2), up = (k == 0 || k == 1);
+    const C fixed = (k == 1 || k == 2) ? C(1) : C(0);
+    const C a = up ? lo[k] : hi[k], b = up ? hi[k] : lo[k];
     const C ax = horiz ? a : fixed, ay = horiz ? fixed : a;
     const C bx = horiz ? b : fixed, by = horiz ? fixed : b;
-    if (any) {
-      // link from the previous interval's end to this start: a chord and its arc
-      twice += xp * ay - ax * yp;
-      const C lx = ax - xp, ly = ay - yp;
-      const C L = vsqrt(lx * lx + ly * ly);
-      if (L > C(0)) seg += segment_area(L < C(2) * R ? L : C(2) * R, R);
-    } else {
-      x0 = ax; y0 = ay;
-      any = true;
-    }
-    twice += ax * by - bx * ay;
-    xp = bx; yp = by;
+    const bool link = on[k] && any;
+    const C lx = add_rn(ax, -xp), ly = add_rn(ay, -yp);
+    l2[k] = link ? fma_rn(lx, lx, mul_rn(ly, ly)) : C(0);
+    C add = link ? fma_rn(xp, ay, -mul_rn(ax, yp)) : C(0);
+    // the interval's own term ax by - bx ay: zero on the edges through (0, 0)
+    if (k == 1 || k == 2) add = add_rn(add, on[k] ? add_rn(hi[k], -lo[k]) : C(0));
+    twice = add_rn(twice, add);
+    x0 = (on[k] && !any) ? ax : x0;
+    y0 = (on[k] && !any) ? ay : y0;
+    xp = on[k] ? bx : xp;
+    yp = on[k] ? by : yp;
+    any = any || on[k];
   }
   if (!any) return C(0);
-  // closing link from the last end back to the first start
-  twice += xp * y0 - x0 * yp;
+  // closing link from the last end back to the first start (l2[0] is free:
+  // no link leads to the first edge)
+  twice = add_rn(twice, fma_rn(xp, y0, -mul_rn(x0, yp)));
   {
-    const C lx = x0 - xp, ly = y0 - yp;
-    const C L = vsqrt(lx * lx + ly * ly);
-    if (L > C(0)) seg += segment_area(L < C(2) * R ? L : C(2) * R, R);
+    const C lx = add_rn(x0, -xp), ly = add_rn(y0, -yp);
+    l2[0] = fma_rn(lx, lx, mul_rn(ly, ly));
   }
-  const C area = C(0.5) * twice + seg;
+  const C most = mul_rn(mul_rn(C(4), R), R);
+  C seg = C(0);
+  for (;;) {  // the links of non-zero length, in the order 1, 2, 3, closing
+    const bool b1 = l2[1] > C(0), b2 = l2[2] > C(0), b3 = l2[3] > C(0);
+    const C L2 = b1 ? l2[1] : (b2 ? l2[2] : (b3 ? l2[3] : l2[0]));
+    if (!(L2 > C(0))) break;
+    if (b1) l2[1] = C(0);
+    else if (b2) l2[2] = C(0);
+    else if (b3) l2[3] = C(0);
+    else l2[0] = C(0);
+    seg = add_rn(seg, segment_area(L2 < most ? L2 : most, R, i2R));
+  }
+  const C area = fma_rn(C(0.5), twice, seg);
   return area < C(0) ? C(0) : (area > C(1) ? C(1) : area);
 }
 
@@ -186,14 +251,18 @@ __host__ __device__ __forceinline__ C disk_unit_cell_area(C cx, C cy, C R) {
 // rounded step by step (mul_rn, add_rn) to come out the same in both.
 enum : int { CELL_BAND = 3 };
 template <class C>
-__host__ __device__ __forceinline__ int quick_class(int il, int jl, const PartTile<C>& p) {
+__host__ __device__ __forceinline__ int quick_class_at(int il, int jl, C xh, C xl, C yh, C yl, C far2, C near2) {
   // centre distance from the cell centre (hi/lo sums keep FP32 exact enough)
-  const C dx = add_rn(add_rn(add_rn(C(il), C(0.5)), -p.xh), -p.xl);
-  const C dy = add_rn(add_rn(add_rn(C(jl), C(0.5)), -p.yh), -p.yl);
+  const C dx = add_rn(add_rn(add_rn(C(il), C(0.5)), -xh), -xl);
+  const C dy = add_rn(add_rn(add_rn(C(jl), C(0.5)), -yh), -yl);
   const C d2 = add_rn(mul_rn(dx, dx), mul_rn(dy, dy));
-  if (d2 >= p.far2) return CELL_FLUID;   // nearest point > R + 0.04
-  if (d2 <= p.near2) return CELL_SOLID;  // farthest corner < R - 0.04
+  if (d2 >= far2) return CELL_FLUID;   // nearest point > R + 0.04
+  if (d2 <= near2) return CELL_SOLID;  // farthest corner < R - 0.04
   return CELL_BAND;
+}
+template <class C>
+__host__ __device__ __forceinline__ int quick_class(int il, int jl, const PartTile<C>& p) {
+  return quick_class_at(il, jl, p.xh, p.xl, p.yh, p.yl, p.far2, p.near2);
 }
 
 // ---------------------------------------------------------------------------
@@ -343,10 +412,17 @@ __host__ __device__ __forceinline__ int cell_fraction(int il, int jl, const Part
   if (cls == CELL_FLUID) { fsp = C(0); return cls; }
   const C cx = (p.xh - C(il)) + p.xl;  // disk centre in cell-local coordinates
   const C cy = (p.yh - C(jl)) + p.yl;
-  fsp = disk_unit_cell_area(cx, cy, p.r);
+  fsp = disk_unit_cell_area(cx, cy, p.r, C(0.5) / p.r);
   return cls;
 }
 
+// A centre coordinate (cell `cells` from the tile's origin, fraction fh + fl)
+// relative to the tile, as an unevaluated sum h + l.
+__host__ __device__ __forceinline__ void tile_coordinate(int cells, float fh, float fl, float& h, float& l) {
+  const float f = float(cells);  // exact small integer
+  h = add_rn(f, fh);
+  l = add_rn(add_rn(add_rn(f, -h), fh), fl);
+}
 // The geometry fields of a particle's raster record as seen from the tile with
 // origin (x0, y0) (FP32, no FP64 arithmetic): everything cell_fraction reads.
 __host__ __device__ __forceinline__ void tile_geometry(const RasterRec& rc, int x0, int y0, PartTile<float>& q) {
@@ -354,13 +430,28 @@ __host__ __device__ __forceinline__ void tile_geometry(const RasterRec& rc, int 
   q.xq = (long long)(rc.xi - x0) * Q + rc.qfx;
   q.yq = (long long)(rc.yi - y0) * Q + rc.qfy;
   q.rq2 = rc.rq2;
-  const float fx = float(rc.xi - x0), fy = float(rc.yi - y0);  // exact small integers
-  q.xh = add_rn(fx, rc.xfh);
-  q.xl = add_rn(add_rn(add_rn(fx, -q.xh), rc.xfh), rc.xfl);
-  q.yh = add_rn(fy, rc.yfh);
-  q.yl = add_rn(add_rn(add_rn(fy, -q.yh), rc.yfh), rc.yfl);
+  tile_coordinate(rc.xi - x0, rc.xfh, rc.xfl, q.xh, q.xl);
+  tile_coordinate(rc.yi - y0, rc.yfh, rc.yfl, q.yh, q.yl);
   q.r = rc.r; q.far2 = rc.far2; q.near2 = rc.near2;
   q.ci = rc.xi; q.cj = rc.yi;
+}
+
+// Class and area of the cell at offset (dx, dy) from the record's own cell
+// against its disk (a band-table entry).  i2R = 1 / (2 R).
+__host__ __device__ __forceinline__ int disk_band_cell(const RasterRec& rc, int dx, int dy, float i2R, float& f) {
+  int cls;
+  if (rc.rq2 < (1ll << 61)) {  // R < 1448 cells: every corner within 2^31 grid units of the centre
+    cls = cell_class_at(dx * (1 << QBITS) - rc.qfx, dy * (1 << QBITS) - rc.qfy, rc.rq2);
+  } else {
+    cls = cell_class_at((long long)dx * (1ll << QBITS) - rc.qfx, (long long)dy * (1ll << QBITS) - rc.qfy, rc.rq2);
+  }
+  if (cls != CELL_INTERFACE) {
+    f = cls == CELL_SOLID ? 1.0f : 0.0f;
+    return cls;
+  }
+  const float cx = add_rn(add_rn(float(-dx), rc.xfh), rc.xfl), cy = add_rn(add_rn(float(-dy), rc.yfh), rc.yfl);
+  f = disk_unit_cell_area(cx, cy, rc.r, i2R);
+  return cls;
 }
 
 }  // namespace vlb
