@@ -32,9 +32,10 @@ lattice_batch_kernel(const BatchLattice<C>* __restrict__ cases, const int* __res
   const TileLists& TL = d.TL[1 - (d.tl ^ par)];
   const int t = blockIdx.x - d.tile0;
   const int tile_y = t / d.K.ntx, tile_x = t - tile_y * d.K.ntx;
-  C f[9], g[9], s_old;
-  pull_direct<S, C, MODE_STEP>(d.K, B, tile_x, tile_y, f, g, s_old);
-  cell_body<S, C, MODE_STEP, HOLD>(d.K, B, d.P, TL, tile_x, tile_y, f, g, s_old, sh,
+  Pair<C> p[9];
+  C s_old;
+  pull_direct<S, C, MODE_STEP>(d.K, B, tile_x, tile_y, p, s_old);
+  cell_body<S, C, MODE_STEP, HOLD>(d.K, B, d.P, TL, tile_x, tile_y, p, s_old, sh,
                                    band_stamp_after(d.stamp, k + 1));
 }
 
@@ -229,9 +230,10 @@ lattice_persistent_kernel(const __grid_constant__ PersistentBatch<C> A) {
       const TileLists& TL = d.TL[1 - (d.tl ^ par)];
       const int lt = item - d.tile0;
       const int tile_y = lt / d.K.ntx, tile_x = lt - tile_y * d.K.ntx;
-      C f[9], g[9], s_old;
-      pull_direct<S, C, MODE_STEP>(d.K, B, tile_x, tile_y, f, g, s_old);
-      cell_body<S, C, MODE_STEP, HOLD>(d.K, B, d.P, TL, tile_x, tile_y, f, g, s_old, sh.tile,
+      Pair<C> p[9];
+      C s_old;
+      pull_direct<S, C, MODE_STEP>(d.K, B, tile_x, tile_y, p, s_old);
+      cell_body<S, C, MODE_STEP, HOLD>(d.K, B, d.P, TL, tile_x, tile_y, p, s_old, sh.tile,
                                        band_stamp_after(d.stamp, s_k + 1));
       __syncthreads();  // every thread's stores and sums of this tile are issued; sh and d are free
       if (tid == 0 && A.with_particles && d.K.np > 0) {

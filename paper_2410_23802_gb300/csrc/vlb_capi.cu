@@ -190,7 +190,8 @@ static void fill_const(vlb_handle* h, LatticeConst<C>& K) {
   // Eq. 5 with the rules of Sec. 3
   const double sp = 1.0 / p.tau_f;
   const double sq = 1.0 / (0.5 + p.lambda_q_flow / (p.tau_f - 0.5));
-  K.s_e = C(p.s_e); K.s_eps = C(p.s_e); K.s_j = C(1); K.s_q = C(sq); K.s_p = C(sp);
+  K.q_e = C(p.s_e / 36.0); K.q_q = C(sq / 12.0); K.q_p = C(sp / 4.0);
+  K.q_fu = C((1.0 - 0.5 * p.s_e) / 6.0); K.q_f4 = C(-(1.0 - 0.5 * sq) / 12.0); K.q_f7 = C(0.5 * (1.0 - 0.5 * sp));
   // Eqs. 11, 22 with rho_f = c_vf = 1; lambda_f = nu / Pr
   const double cvf = 1.0, cvs = p.cv_ratio;
   const double cref = 2.0 * cvf * cvs / (cvf + cvs);
@@ -520,16 +521,26 @@ vlb_status vlb_add_ellipses(vlb_handle* h, int32_t n, const double* xy, const do
   return VLB_OK;
 }
 
-// Lattice pass with list buffer `lists`; STEP and INIT also clear the other
-// list buffer for the next particle step.
-static vlb_status launch_lattice(vlb_handle* h, int mode, int src_buf, int dst_buf, int lists) {
+// The buffers of a pass from population buffer src_buf into dst_buf.
+static StepBuffers step_buffers(const vlb_handle* h, int src_buf, int dst_buf) {
   StepBuffers B;
-  B.src = h->pop[src_buf];
-  B.dst = h->pop[dst_buf];
+  const long long pair = 2 * (long long)h->ssize;
+  for (int i = 0; i < 9; ++i) {
+    B.plane[i] = static_cast<const char*>(h->pop[src_buf]) + i * h->plane * pair;
+    B.pull[i] = B.plane[i] - (ex(i) + (long long)ey(i) * h->pitch) * pair;
+    B.dst[i] = static_cast<char*>(h->pop[dst_buf]) + i * h->plane * pair;
+  }
   B.s_src = h->spl[src_buf];
   B.s_dst = h->spl[dst_buf];
   B.macro = h->macro;
   B.err = h->err_dev;
+  return B;
+}
+
+// Lattice pass with list buffer `lists`; STEP and INIT also clear the other
+// list buffer for the next particle step.
+static vlb_status launch_lattice(vlb_handle* h, int mode, int src_buf, int dst_buf, int lists) {
+  const StepBuffers B = step_buffers(h, src_buf, dst_buf);
   TileLists TL = h->TL[lists];
   TL.next_count = mode == MODE_MACROS ? nullptr : h->TL[1 - lists].count;
   cudaError_t e = h->p.precision == VLB_FP64 ? launch_lattice_f64(mode, h->K64, B, h->P, TL, h->stream)
@@ -541,7 +552,7 @@ static vlb_status launch_lattice(vlb_handle* h, int mode, int src_buf, int dst_b
 // Each band-kernel pass writes its entries with a new stamp (1 .. 2^29 - 1,
 // cycling); the lattice and dump kernels accept only entries with the stamp of
 // the tables they are given.
-static void advance_band_stamp(vlb_handle* h, long long levels) {
+static void advance_band_stamp(vlb_handle* h, int levels) {
   const int s = band_stamp_after(h->PC.band_stamp, levels);
   h->PC.band_stamp = s;
   h->K32.band_stamp = h->K64.band_stamp = s;
@@ -823,12 +834,7 @@ void fill_lattice_desc(vlb_handle* h, const LatticeConst<C>& K, int tile0, Batch
   d = BatchLattice<C>{};
   d.K = K;
   for (int b = 0; b < 2; ++b) {
-    d.B[b].src = h->pop[b];
-    d.B[b].dst = h->pop[1 - b];
-    d.B[b].s_src = h->spl[b];
-    d.B[b].s_dst = h->spl[1 - b];
-    d.B[b].macro = h->macro;
-    d.B[b].err = h->err_dev;
+    d.B[b] = step_buffers(h, b, 1 - b);
     d.TL[b] = h->TL[b];
     d.TL[b].next_count = h->TL[1 - b].count;
   }
@@ -1388,7 +1394,9 @@ vlb_status vlb_get_contact_pairs(vlb_handle* h, int32_t capacity, int32_t* pairs
 
 // ---- checkpoint and resume -------------------------------------------------
 // The image is a header followed by the device buffers that carry the state
-// of the current level, byte for byte: both population buffers and S planes
+// of the current level, byte for byte but for the populations, which are
+// written as eighteen planes (f_0 .. f_8, g_0 .. g_8) rather than as the nine
+// planes of pairs they are on the device: both population buffers and S planes
 // (the field read-back re-runs the last step's pre-collision part from the
 // previous one), the particle block (state, constants, records, ranges,
 // contact lists), the exchange accumulators, the band tables and both tile
@@ -1431,6 +1439,67 @@ uint64_t state_bytes(const StateHeader& H) {
 }
 }  // namespace
 
+}  // extern "C"
+
+// Population buffer b to (out) or from (in) an image's eighteen planes, a
+// direction at a time: split or joined on the device in two planes of scratch,
+// or on the host where the device has no room for them.
+template <class W>
+static void split_on_host(W* pairs, W* f, W* g, size_t n, bool join) {
+  for (size_t c = 0; c < n; ++c) {
+    if (join) {
+      pairs[2 * c] = f[c];
+      pairs[2 * c + 1] = g[c];
+    } else {
+      f[c] = pairs[2 * c];
+      g[c] = pairs[2 * c + 1];
+    }
+  }
+}
+static cudaError_t copy_populations(vlb_handle* h, int b, char* out, const char* in) {
+  const size_t n = (size_t)h->plane, plane = n * h->ssize;
+  char* scratch = nullptr;
+  cudaError_t e = cudaMalloc(reinterpret_cast<void**>(&scratch), 2 * plane);
+  if (e == cudaErrorMemoryAllocation) {
+    cudaGetLastError();
+    std::vector<char> pairs(2 * plane), two(2 * plane);
+    auto split = [&](bool join) {
+      char *q = pairs.data(), *f = two.data(), *g = f + plane;
+      if (h->ssize == 8) split_on_host((uint64_t*)q, (uint64_t*)f, (uint64_t*)g, n, join);
+      else if (h->ssize == 4) split_on_host((uint32_t*)q, (uint32_t*)f, (uint32_t*)g, n, join);
+      else split_on_host((uint16_t*)q, (uint16_t*)f, (uint16_t*)g, n, join);
+    };
+    e = cudaSuccess;
+    for (int i = 0; i < 9 && e == cudaSuccess; ++i) {
+      char* dev = static_cast<char*>(h->pop[b]) + 2 * plane * i;
+      if (in) {
+        for (int q = 0; q < 2; ++q) std::memcpy(two.data() + q * plane, in + (9 * q + i) * plane, plane);
+        split(true);
+        e = cudaMemcpy(dev, pairs.data(), 2 * plane, cudaMemcpyHostToDevice);
+      } else {
+        e = cudaMemcpy(pairs.data(), dev, 2 * plane, cudaMemcpyDeviceToHost);
+        split(false);
+        for (int q = 0; q < 2; ++q) std::memcpy(out + (9 * q + i) * plane, two.data() + q * plane, plane);
+      }
+    }
+    return e;
+  }
+  for (int i = 0; i < 9 && e == cudaSuccess; ++i) {
+    char* pairs = static_cast<char*>(h->pop[b]) + 2 * plane * i;
+    for (int q = 0; q < 2 && in && e == cudaSuccess; ++q)
+      e = cudaMemcpy(scratch + q * plane, in + (9 * q + i) * plane, plane, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess)
+      e = launch_split_plane(pairs, scratch, scratch + plane, h->plane, h->ssize, in != nullptr, h->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+    for (int q = 0; q < 2 && out && e == cudaSuccess; ++q)
+      e = cudaMemcpy(out + (9 * q + i) * plane, scratch + q * plane, plane, cudaMemcpyDeviceToHost);
+  }
+  cudaFree(scratch);
+  return e;
+}
+
+extern "C" {
+
 vlb_status vlb_state_size(vlb_handle* h, uint64_t* bytes) {
   if (!h || !bytes) return VLB_EINVAL;
   vlb_status s;
@@ -1456,7 +1525,8 @@ vlb_status vlb_save_state(vlb_handle* h, void* buf, uint64_t bytes) {
     return e;
   };
   for (int b = 0; b < 2; ++b) {
-    CK(h, get(h->pop[b], H.pop_bytes));
+    CK(h, copy_populations(h, b, o, nullptr));
+    o += H.pop_bytes;
     CK(h, get(h->spl[b], H.s_bytes));
   }
   CK(h, get(h->pbase, H.part_bytes));
@@ -1494,7 +1564,8 @@ vlb_status vlb_load_state(vlb_handle* h, const void* buf, uint64_t bytes) {
     return e;
   };
   for (int b = 0; b < 2; ++b) {
-    CK(h, put(h->pop[b], I.pop_bytes));
+    CK(h, copy_populations(h, b, nullptr, o));
+    o += I.pop_bytes;
     CK(h, put(h->spl[b], I.s_bytes));
   }
   CK(h, put(h->pbase, I.part_bytes));

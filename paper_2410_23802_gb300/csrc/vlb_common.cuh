@@ -58,8 +58,9 @@ enum : unsigned {
 // Band-table stamps run 1 .. 2^29 - 1 and then start again at 1 (0: none
 // yet); the stamp k >= 1 levels after stamp s.
 constexpr int BAND_STAMP_CYCLE = (1 << 29) - 1;
-__host__ __device__ __forceinline__ int band_stamp_after(int s, long long k) {
-  return 1 + (int)(((long long)s - 1 + k) % BAND_STAMP_CYCLE);
+__host__ __device__ __forceinline__ int band_stamp_after(int s, int k) {
+  // (32 bits hold s - 1 + k, and a 64-bit remainder is a subroutine on the device)
+  return 1 + (int)(((unsigned)(s - 1) + (unsigned)k) % (unsigned)BAND_STAMP_CYCLE);
 }
 
 // Kernel modes of the lattice kernel.
@@ -163,8 +164,10 @@ struct LatticeConst {
   double zeta;             // contact range
   double contact_scale;    // |rho_r - 1| rho_f |g| pi
   double eps_p;            // particle-particle stiffness parameter
-  // flow rates (Eq. 5)
-  C s_e, s_eps, s_j, s_q, s_p;
+  // flow rates (Eq. 5) times the factors of M^-1, s_e = s_eps: s_e / 36,
+  // s_q / 12, s_p / 4, and the forcing's (1 - s_e / 2) / 6, -(1 - s_q / 2) / 12,
+  // (1 - s_p / 2) / 2
+  C q_e, q_q, q_p, q_fu, q_f4, q_f7;
   // thermal (Eqs. 11, 18-22)
   C cv_f, cv_s, cref, lam_f, rates_mode;
   C bx, by, T_ref, T_fluid;  // buoyancy b = -rho_f beta g; T_f = initial fluid temperature
@@ -175,8 +178,13 @@ struct LatticeConst {
 };
 
 struct StepBuffers {
-  void* src;     // populations at level n (18 planes of the storage type)
-  void* dst;     // populations at level n+1
+  // Planes of (f, g) pairs of the storage type, as one pointer per direction,
+  // so that an entry's address is one multiply-add of the cell index (the
+  // kernel's own 64-bit products of plane sizes were a fifth of its
+  // instructions).
+  const char* pull[9];   // level n: plane i shifted by -e_i (the entry that an interior cell pulls)
+  const char* plane[9];  // level n: plane i
+  char* dst[9];          // level n+1: plane i
   void* s_src;   // S = 2 f_s + df_s/dt at level n (one plane, arithmetic type)
   void* s_dst;
   void* macro;   // rho, ux, uy, T, fs planes (arithmetic type); may be null

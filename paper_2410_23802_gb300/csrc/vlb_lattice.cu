@@ -8,9 +8,10 @@ template <class S, class C, int MODE, bool HOLD>
 __global__ void __launch_bounds__(TILE_X * TILE_Y, sizeof(C) == 4 ? VLB_LATTICE_MIN_BLOCKS : 1)
 lattice_kernel(const LatticeConst<C> K, const StepBuffers B, const ParticleArrays P, const TileLists TL) {
   __shared__ TileShared<C> sh;
-  C f[9], g[9], s_old;
-  pull_direct<S, C, MODE>(K, B, blockIdx.x, blockIdx.y, f, g, s_old);
-  cell_body<S, C, MODE, HOLD>(K, B, P, TL, blockIdx.x, blockIdx.y, f, g, s_old, sh, K.band_stamp);
+  Pair<C> p[9];
+  C s_old;
+  pull_direct<S, C, MODE>(K, B, blockIdx.x, blockIdx.y, p, s_old);
+  cell_body<S, C, MODE, HOLD>(K, B, P, TL, blockIdx.x, blockIdx.y, p, s_old, sh, K.band_stamp);
 }
 
 // Ownership of every cell at the current level, from the same raster code as
@@ -42,8 +43,8 @@ raster_dump_kernel(const LatticeConst<C> K, const ParticleArrays P, const TileLi
 // deviations from w_i, so each cell adds 1), eps and g (macro planes 5, 6),
 // then one ordered pass over the block sums.
 template <class S, class C>
-__global__ void audit_blocks_kernel(const LatticeConst<C> K, const S* pop, const C* macro, double* scratch,
-                                    unsigned* err) {
+__global__ void audit_blocks_kernel(const LatticeConst<C> K, const typename StoredPair<S>::type* pop, const C* macro,
+                                    double* scratch, unsigned* err) {
   __shared__ double red[3][256];
   double sf = 0.0, se = 0.0, sg = 0.0;
   bool bad = false;
@@ -54,8 +55,9 @@ __global__ void audit_blocks_kernel(const LatticeConst<C> K, const S* pop, const
     const long long cell = y * K.pitch + x;
     double cf = 1.0;
     for (int i = 0; i < 9; ++i) {
-      const double v = double(stored_value<float, S>(pop[(long long)i * K.plane + cell]));
-      const double w = double(stored_value<float, S>(pop[(long long)(9 + i) * K.plane + cell]));
+      const typename StoredPair<S>::type fg = pop[(long long)i * K.plane + cell];
+      const double v = double(stored_value<float, S>(fg.x));
+      const double w = double(stored_value<float, S>(fg.y));
       bad |= !(v == v) || !(w == w);
       cf += v;
     }
@@ -129,7 +131,7 @@ cudaError_t launch_raster_dump_f64(const LatticeConst<double>& K, const Particle
 template <class S, class C>
 static cudaError_t audit(const LatticeConst<C>& K, const void* pop, const void* macro, double* scratch,
                          int nblocks, double* out, unsigned* err, cudaStream_t st) {
-  audit_blocks_kernel<S, C><<<nblocks, 256, 0, st>>>(K, static_cast<const S*>(pop),
+  audit_blocks_kernel<S, C><<<nblocks, 256, 0, st>>>(K, static_cast<const typename StoredPair<S>::type*>(pop),
                                                      static_cast<const C*>(macro), scratch, err);
   audit_final_kernel<<<1, 32, 0, st>>>(scratch, nblocks, out);
   return cudaGetLastError();
@@ -143,6 +145,31 @@ cudaError_t launch_audit_f32(const LatticeConst<float>& K, const void* pop, cons
 cudaError_t launch_audit_f64(const LatticeConst<double>& K, const void* pop, const void* macro,
                              double* scratch, int nblocks, double* out, unsigned* err, cudaStream_t st) {
   return audit<double, double>(K, pop, macro, scratch, nblocks, out, err, st);
+}
+
+// One plane of (f_i, g_i) pairs to or from its two planes f_i, g_i (the form
+// of a state image); W: an unsigned word of a population's size.
+template <class W>
+__global__ void split_plane_kernel(W* __restrict__ pairs, W* __restrict__ f, W* __restrict__ g, long long n, int join) {
+  for (long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x; c < n; c += (long long)gridDim.x * blockDim.x) {
+    if (join) {
+      pairs[2 * c] = f[c];
+      pairs[2 * c + 1] = g[c];
+    } else {
+      f[c] = pairs[2 * c];
+      g[c] = pairs[2 * c + 1];
+    }
+  }
+}
+template <class W>
+static cudaError_t split(void* pairs, void* f, void* g, long long n, bool join, cudaStream_t st) {
+  split_plane_kernel<W><<<608, 256, 0, st>>>(static_cast<W*>(pairs), static_cast<W*>(f), static_cast<W*>(g), n, join);
+  return cudaGetLastError();
+}
+cudaError_t launch_split_plane(void* pairs, void* f, void* g, long long n, size_t bytes, bool join, cudaStream_t st) {
+  if (bytes == 8) return split<unsigned long long>(pairs, f, g, n, join, st);
+  if (bytes == 4) return split<unsigned>(pairs, f, g, n, join, st);
+  return split<unsigned short>(pairs, f, g, n, join, st);
 }
 
 }  // namespace vlb
