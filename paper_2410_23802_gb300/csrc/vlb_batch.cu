@@ -12,31 +12,54 @@
 namespace vlb {
 
 // Step k of a batch call (vlb_step_batch) over the tiles of many cases, one
-// CTA per tile: the tile's case descriptor is copied to shared memory, then
-// the single-case code (vlb_lattice_body.cuh) runs on it.
+// CTA per tile (FP64: per strip of a tile): the tile's case descriptor is
+// copied to shared memory, then the single-case code (vlb_lattice_body.cuh)
+// runs on it.  The first `duty` CTAs have the once-per-tile work, a lane per
+// tile (tile_duties).
 template <class S, class C, bool HOLD>
-__global__ void __launch_bounds__(TILE_X * TILE_Y, sizeof(C) == 4 ? VLB_LATTICE_MIN_BLOCKS : 1)
-lattice_batch_kernel(const BatchLattice<C>* __restrict__ cases, const int* __restrict__ tile_case, int k) {
-  __shared__ TileShared<C> sh;
+__global__ void __launch_bounds__(32 * tile_warps<C>(), sizeof(C) == 4 ? VLB_LATTICE_MIN_BLOCKS : 1)
+lattice_batch_kernel(const BatchLattice<C>* __restrict__ cases, const int* __restrict__ tile_case, int ntiles, int k,
+                     int duty) {
+  constexpr int WARPS = tile_warps<C>(), PARTS = TILE_Y / WARPS;
+  __shared__ PartTile<C> list[WARPS][TILE_CAP];
   __shared__ BatchLattice<C> d;
   static_assert(sizeof(BatchLattice<C>) % 4 == 0, "descriptor copied as words");
+  const int lane = threadIdx.x, warp = threadIdx.y, par = k & 1;
+  if (blockIdx.x < duty) {
+    const int span = duty_span(ntiles), first = span * (blockIdx.x * WARPS + warp), t = first + lane;
+    int n = 0, c = 0;
+    if (lane < span && t < ntiles) {
+      c = tile_case[t];
+      const BatchLattice<C>& e = cases[c];
+      const TileLists& TL = e.TL[1 - (e.tl ^ par)];
+      n = min(TL.count[t - e.tile0], TILE_CAP);
+      TL.next_count[t - e.tile0] = 0;
+    }
+    for (unsigned m = __ballot_sync(0xffffffffu, n > 1); m; m &= m - 1) {
+      const int l = __ffs(m) - 1;
+      const BatchLattice<C>& e = cases[__shfl_sync(0xffffffffu, c, l)];
+      contact_pairs(e.K, e.P, e.TL[1 - (e.tl ^ par)].ids, __shfl_sync(0xffffffffu, n, l), first + l - e.tile0, lane,
+                    e.B[0].err);
+    }
+    return;
+  }
+  const int block = blockIdx.x - duty, tile = block / PARTS;
   {
-    const int* src = reinterpret_cast<const int*>(cases + tile_case[blockIdx.x]);
+    const int* src = reinterpret_cast<const int*>(cases + tile_case[tile]);
     int* dst = reinterpret_cast<int*>(&d);
-    for (int w = threadIdx.y * TILE_X + threadIdx.x; w < (int)(sizeof(d) / 4); w += TILE_X * TILE_Y)
-      dst[w] = src[w];
+    for (int w = 32 * warp + lane; w < (int)(sizeof(d) / 4); w += 32 * WARPS) dst[w] = src[w];
   }
   __syncthreads();
-  const int par = k & 1;
   const StepBuffers& B = d.B[d.cur ^ par];
-  const TileLists& TL = d.TL[1 - (d.tl ^ par)];
-  const int t = blockIdx.x - d.tile0;
+  const int t = tile - d.tile0;
   const int tile_y = t / d.K.ntx, tile_x = t - tile_y * d.K.ntx;
+  const CellAt at = cell_at<S>(tile_x, tile_y, WARPS == 1 ? block % PARTS : warp, lane);
+  if (WARPS == 1 && tile_x * TILE_X + at.bx >= d.K.nx) return;  // a strip beyond the lattice
+  const ListHead head = list_head(d.TL[1 - (d.tl ^ par)], t, lane);
   Pair<C> p[9];
   C s_old;
-  pull_direct<S, C, MODE_STEP>(d.K, B, tile_x, tile_y, p, s_old);
-  cell_body<S, C, MODE_STEP, HOLD>(d.K, B, d.P, TL, tile_x, tile_y, p, s_old, sh,
-                                   band_stamp_after(d.stamp, k + 1));
+  pull_direct<S, C, MODE_STEP>(d.K, B, at, p, s_old);
+  cell_body<S, C, MODE_STEP, HOLD>(d.K, B, d.P, at, head, p, s_old, list[warp], band_stamp_after(d.stamp, k + 1));
 }
 
 // The same over the particles of many cases, step k of a batch call; `group`
@@ -70,9 +93,12 @@ template <class S, class C>
 static cudaError_t launch_batch(const BatchLattice<C>* cases, const int* tile_case, int ntiles, int k, bool held,
                                 cudaStream_t st) {
   if (ntiles == 0) return cudaSuccess;
-  const dim3 block(TILE_X, TILE_Y);
-  if (held) lattice_batch_kernel<S, C, true><<<(unsigned)ntiles, block, 0, st>>>(cases, tile_case, k);
-  else lattice_batch_kernel<S, C, false><<<(unsigned)ntiles, block, 0, st>>>(cases, tile_case, k);
+  constexpr int WARPS = tile_warps<C>();
+  const dim3 block(32, WARPS);
+  const int per_cta = duty_span(ntiles) * WARPS, duty = (ntiles + per_cta - 1) / per_cta;
+  const unsigned grid = (unsigned)duty + (unsigned)ntiles * (TILE_Y / WARPS);
+  if (held) lattice_batch_kernel<S, C, true><<<grid, block, 0, st>>>(cases, tile_case, ntiles, k, duty);
+  else lattice_batch_kernel<S, C, false><<<grid, block, 0, st>>>(cases, tile_case, ntiles, k, duty);
   return cudaGetLastError();
 }
 
@@ -182,8 +208,8 @@ __global__ void __launch_bounds__(TILE_X * TILE_Y, sizeof(C) == 4 ? VLB_LATTICE_
 lattice_persistent_kernel(const __grid_constant__ PersistentBatch<C> A) {
   constexpr int NWARPS = TILE_X * TILE_Y / 32;
   union Shared {
-    TileShared<C> tile;             // a tile's particles
-    int queue[NWARPS][BAND_QUEUE];  // the band queues of a particle group
+    PartTile<C> list[NWARPS][TILE_CAP];  // the particles of each warp's block
+    int queue[NWARPS][BAND_QUEUE];       // the band queues of a particle group
   };
   __shared__ Shared sh;
   __shared__ BatchLattice<C> d;
@@ -230,11 +256,18 @@ lattice_persistent_kernel(const __grid_constant__ PersistentBatch<C> A) {
       const TileLists& TL = d.TL[1 - (d.tl ^ par)];
       const int lt = item - d.tile0;
       const int tile_y = lt / d.K.ntx, tile_x = lt - tile_y * d.K.ntx;
+      const int lane = threadIdx.x, warp = threadIdx.y;
+      const CellAt at = cell_at<S>(tile_x, tile_y, warp, lane);
+      const ListHead head = list_head(TL, lt, lane);
       Pair<C> p[9];
       C s_old;
-      pull_direct<S, C, MODE_STEP>(d.K, B, tile_x, tile_y, p, s_old);
-      cell_body<S, C, MODE_STEP, HOLD>(d.K, B, d.P, TL, tile_x, tile_y, p, s_old, sh.tile,
+      pull_direct<S, C, MODE_STEP>(d.K, B, at, p, s_old);
+      cell_body<S, C, MODE_STEP, HOLD>(d.K, B, d.P, at, head, p, s_old, sh.list[warp],
                                        band_stamp_after(d.stamp, s_k + 1));
+      if (warp == 0) {
+        if (lane == 0) TL.next_count[lt] = 0;  // the next particle step fills the other list buffer
+        if (head.count > 1) contact_pairs(d.K, d.P, TL.ids, head.count, lt, lane, B.err);
+      }
       __syncthreads();  // every thread's stores and sums of this tile are issued; sh and d are free
       if (tid == 0 && A.with_particles && d.K.np > 0) {
         // counted now, published (fence + add) when the case changes or the

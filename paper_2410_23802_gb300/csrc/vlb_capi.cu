@@ -190,7 +190,7 @@ static void fill_const(vlb_handle* h, LatticeConst<C>& K) {
   // Eq. 5 with the rules of Sec. 3
   const double sp = 1.0 / p.tau_f;
   const double sq = 1.0 / (0.5 + p.lambda_q_flow / (p.tau_f - 0.5));
-  K.q_e = C(p.s_e / 36.0); K.q_q = C(sq / 12.0); K.q_p = C(sp / 4.0);
+  K.q_e = C(p.s_e / 4.0); K.q_q = C(sq / 12.0); K.q_p = C(sp / 4.0);
   K.q_fu = C((1.0 - 0.5 * p.s_e) / 6.0); K.q_f4 = C(-(1.0 - 0.5 * sq) / 12.0); K.q_f7 = C(0.5 * (1.0 - 0.5 * sp));
   // Eqs. 11, 22 with rho_f = c_vf = 1; lambda_f = nu / Pr
   const double cvf = 1.0, cvs = p.cv_ratio;

@@ -164,9 +164,9 @@ struct LatticeConst {
   double zeta;             // contact range
   double contact_scale;    // |rho_r - 1| rho_f |g| pi
   double eps_p;            // particle-particle stiffness parameter
-  // flow rates (Eq. 5) times the factors of M^-1, s_e = s_eps: s_e / 36,
-  // s_q / 12, s_p / 4, and the forcing's (1 - s_e / 2) / 6, -(1 - s_q / 2) / 12,
-  // (1 - s_p / 2) / 2
+  // flow rates (Eq. 5) times the factors they meet in the collision, s_e =
+  // s_eps: s_e / 4, s_q / 12, s_p / 4, and the forcing's (1 - s_e / 2) / 6,
+  // -(1 - s_q / 2) / 12, (1 - s_p / 2) / 2
   C q_e, q_q, q_p, q_fu, q_f4, q_f7;
   // thermal (Eqs. 11, 18-22)
   C cv_f, cv_s, cref, lam_f, rates_mode;

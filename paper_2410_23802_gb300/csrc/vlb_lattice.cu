@@ -4,14 +4,32 @@
 
 namespace vlb {
 
+// One CTA per tile (FP32: TILE_Y warps), or per strip of a tile (FP64: one
+// warp per CTA, grid ntx * TILE_Y across).  FP64 arithmetic bounds the FP64
+// kernel (a warp's FP64 instruction takes the SM about 16 cycles whether one
+// lane needs it or 32), so its warps are spread evenly over the SMs and kept
+// full: on a 100 x 400 channel, tiles of four warps put three CTAs on some SMs
+// and two on others and gave the fourth tile column 4 live lanes in 32.
+// The first `duty` rows of the grid have the once-per-tile work (tile_duties).
 template <class S, class C, int MODE, bool HOLD>
-__global__ void __launch_bounds__(TILE_X * TILE_Y, sizeof(C) == 4 ? VLB_LATTICE_MIN_BLOCKS : 1)
-lattice_kernel(const LatticeConst<C> K, const StepBuffers B, const ParticleArrays P, const TileLists TL) {
-  __shared__ TileShared<C> sh;
+__global__ void __launch_bounds__(32 * tile_warps<C>(), sizeof(C) == 4 ? VLB_LATTICE_MIN_BLOCKS : 1)
+lattice_kernel(const LatticeConst<C> K, const StepBuffers B, const ParticleArrays P, const TileLists TL, int duty) {
+  constexpr int WARPS = tile_warps<C>();
+  __shared__ PartTile<C> list[WARPS][TILE_CAP];
+  const int lane = threadIdx.x, warp = threadIdx.y;
+  if (blockIdx.y < duty) {
+    const int ntiles = K.ntx * K.nty, span = duty_span(ntiles);
+    tile_duties(K, P, TL, span * ((blockIdx.y * gridDim.x + blockIdx.x) * WARPS + warp), span, ntiles, lane, B.err);
+    return;
+  }
+  const int tile_x = blockIdx.x / (TILE_Y / WARPS), tile_y = blockIdx.y - duty;
+  const CellAt at = cell_at<S>(tile_x, tile_y, WARPS == 1 ? blockIdx.x % TILE_Y : warp, lane);
+  if (WARPS == 1 && tile_x * TILE_X + at.bx >= K.nx) return;  // a strip beyond the lattice
+  const ListHead head = list_head(TL, tile_y * K.ntx + tile_x, lane);
   Pair<C> p[9];
   C s_old;
-  pull_direct<S, C, MODE>(K, B, blockIdx.x, blockIdx.y, p, s_old);
-  cell_body<S, C, MODE, HOLD>(K, B, P, TL, blockIdx.x, blockIdx.y, p, s_old, sh, K.band_stamp);
+  pull_direct<S, C, MODE>(K, B, at, p, s_old);
+  cell_body<S, C, MODE, HOLD>(K, B, P, at, head, p, s_old, list[warp], K.band_stamp);
 }
 
 // Ownership of every cell at the current level, from the same raster code as
@@ -20,24 +38,35 @@ template <class C>
 __global__ void __launch_bounds__(TILE_X * TILE_Y)
 raster_dump_kernel(const LatticeConst<C> K, const ParticleArrays P, const TileLists TL, unsigned char* count,
                    int* owner, unsigned char* flag, double* fsp, unsigned* err) {
-  __shared__ TileShared<C> sh;
-  const int tx = threadIdx.x, ty = threadIdx.y;
-  const int np = load_tile_particles<C>(K, P, TL, blockIdx.x, blockIdx.y, sh);
-  const int x = blockIdx.x * TILE_X + tx, y = blockIdx.y * TILE_Y + ty;
+  __shared__ PartTile<C> lists[TILE_Y][TILE_CAP];
+  const CellAt at = cell_at<float>(blockIdx.x, blockIdx.y, threadIdx.y, threadIdx.x);
+  PartTile<C>* list = lists[threadIdx.y];
+  const ListHead head = list_head(TL, at.tile_y * K.ntx + at.tile_x, at.lane);
+  const int np = load_block_particles<float, C>(P, head, at, false, list);
+  const int x = at.tile_x * TILE_X + at.tx, y = at.tile_y * TILE_Y + at.ty;
   if (x >= K.nx || y >= K.ny) return;
-  int nown, own[MAX_OWNERS], cls[MAX_OWNERS];
-  C ofs[MAX_OWNERS];
-  const PartTile<C>* s_p = sh.p;
-  raster_cell<C>(tx, ty, x, y, np, s_p, P.band, K.band_off, K.band_stamp, nown, own, cls, ofs, err);
+  int nown = 0, own[MAX_OWNERS] = {-1, -1, -1, -1}, cls[MAX_OWNERS] = {};
+  C ofs[MAX_OWNERS] = {}, fs = C(0);
+  for (int s = 0; s < np; ++s) {
+    C f;
+    const int c = particle_share(list[s], at.tx, at.ty, x, y, P.band, K.band_off, K.band_stamp, f, err);
+    if (c == CELL_FLUID) continue;
+    if (nown == MAX_OWNERS) { atomicOr(err, ERR_OWNER_OVERFLOW); break; }
+    own[nown] = list[s].id;
+    cls[nown] = c;
+    ofs[nown++] = f;
+    fs += f;
+  }
+  const C scale = fs > C(1) ? C(1) / fs : C(1);
   const long long c = (long long)y * K.nx + x;
   count[c] = (unsigned char)nown;
-#pragma unroll
   for (int k = 0; k < MAX_OWNERS; ++k) {
-    owner[4 * c + k] = k < nown ? s_p[own[k]].id : -1;
-    flag[4 * c + k] = (unsigned char)(k < nown ? cls[k] : 0);
-    fsp[4 * c + k] = k < nown ? double(ofs[k]) : 0.0;
+    owner[4 * c + k] = own[k];
+    flag[4 * c + k] = (unsigned char)cls[k];
+    fsp[4 * c + k] = double(ofs[k] * scale);
   }
 }
+static_assert(MAX_OWNERS == 4, "four owners per cell in the dump");
 
 // FP64 audit of the stored state: per-block sums of f (populations are
 // deviations from w_i, so each cell adds 1), eps and g (macro planes 5, 6),
@@ -88,13 +117,19 @@ __global__ void audit_final_kernel(const double* scratch, int nblocks, double* o
 template <class S, class C>
 static cudaError_t launch_mode(int mode, const LatticeConst<C>& K, const StepBuffers& B,
                                const ParticleArrays& P, const TileLists& TL, cudaStream_t st) {
-  dim3 grid(K.ntx, K.nty), block(TILE_X, TILE_Y);
+  constexpr int WARPS = tile_warps<C>();
+  const int across = K.ntx * (TILE_Y / WARPS);
+  // rows of CTAs for the once-per-tile work
+  const int ntiles = K.ntx * K.nty, per_cta = duty_span(ntiles) * WARPS;
+  const int duty_ctas = (ntiles + per_cta - 1) / per_cta;
+  const int duty = mode != MODE_MACROS && K.np > 0 ? (duty_ctas + across - 1) / across : 0;
+  const dim3 grid(across, K.nty + duty), block(32, WARPS);
   // kernels with the held-temperature path only where some particle is held
-  if (mode == MODE_INIT) lattice_kernel<S, C, MODE_INIT, false><<<grid, block, 0, st>>>(K, B, P, TL);
-  else if (mode == MODE_STEP && K.any_held) lattice_kernel<S, C, MODE_STEP, true><<<grid, block, 0, st>>>(K, B, P, TL);
-  else if (mode == MODE_STEP) lattice_kernel<S, C, MODE_STEP, false><<<grid, block, 0, st>>>(K, B, P, TL);
-  else if (K.any_held) lattice_kernel<S, C, MODE_MACROS, true><<<grid, block, 0, st>>>(K, B, P, TL);
-  else lattice_kernel<S, C, MODE_MACROS, false><<<grid, block, 0, st>>>(K, B, P, TL);
+  if (mode == MODE_INIT) lattice_kernel<S, C, MODE_INIT, false><<<grid, block, 0, st>>>(K, B, P, TL, duty);
+  else if (mode == MODE_STEP && K.any_held) lattice_kernel<S, C, MODE_STEP, true><<<grid, block, 0, st>>>(K, B, P, TL, duty);
+  else if (mode == MODE_STEP) lattice_kernel<S, C, MODE_STEP, false><<<grid, block, 0, st>>>(K, B, P, TL, duty);
+  else if (K.any_held) lattice_kernel<S, C, MODE_MACROS, true><<<grid, block, 0, st>>>(K, B, P, TL, duty);
+  else lattice_kernel<S, C, MODE_MACROS, false><<<grid, block, 0, st>>>(K, B, P, TL, duty);
   return cudaGetLastError();
 }
 

@@ -90,7 +90,6 @@ struct PartTile : EllPart<C> {
   int id;                 // particle id
   int ci, cj;             // cell of the centre (band table origin)
   int fixed;              // held at T0: 1 covered part (reading R11), 2 whole cells (R11b)
-  int rx, ry;             // first tile of the particle's range
 };
 
 // Class of the cell whose lower-left corner lies at (cx0, cy0) from the disk's
