@@ -24,6 +24,7 @@ lattice_batch_kernel(const BatchLattice<C>* __restrict__ cases, const int* __res
   __shared__ PartTile<C> list[WARPS][TILE_CAP];
   __shared__ BatchLattice<C> d;
   static_assert(sizeof(BatchLattice<C>) % 4 == 0, "descriptor copied as words");
+  begin_chained();
   const int lane = threadIdx.x, warp = threadIdx.y, par = k & 1;
   if (blockIdx.x < duty) {
     const int span = duty_span(ntiles), first = span * (blockIdx.x * WARPS + warp), t = first + lane;
@@ -68,6 +69,7 @@ __global__ void __launch_bounds__(STEP_THREADS)
     particle_step_batch_kernel(const BatchParticles* __restrict__ cases, const int2* __restrict__ items, int nitems,
                                int k, int group) {
   __shared__ StepShared sh;
+  begin_chained();
   const int i0 = blockIdx.x * group;
   step_group(min(group, nitems - i0), [&](int s) {
     const int2 it = items[i0 + s];
@@ -80,6 +82,7 @@ __global__ void __launch_bounds__(32 * ELL_WARPS)
     particle_ellipse_batch_kernel(const BatchParticles* __restrict__ cases, const int2* __restrict__ items, int blocks,
                                   int k, const int* __restrict__ kdev) {
   __shared__ int s_queue[ELL_WARPS][32];
+  begin_chained();
   if (kdev) k = *kdev;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int i = blockIdx.x / blocks, by = (blockIdx.x - i * blocks) * ELL_WARPS + warp;
@@ -97,9 +100,8 @@ static cudaError_t launch_batch(const BatchLattice<C>* cases, const int* tile_ca
   const dim3 block(32, WARPS);
   const int per_cta = duty_span(ntiles) * WARPS, duty = (ntiles + per_cta - 1) / per_cta;
   const unsigned grid = (unsigned)duty + (unsigned)ntiles * (TILE_Y / WARPS);
-  if (held) lattice_batch_kernel<S, C, true><<<grid, block, 0, st>>>(cases, tile_case, ntiles, k, duty);
-  else lattice_batch_kernel<S, C, false><<<grid, block, 0, st>>>(cases, tile_case, ntiles, k, duty);
-  return cudaGetLastError();
+  return launch_chained(held ? lattice_batch_kernel<S, C, true> : lattice_batch_kernel<S, C, false>, dim3(grid), block,
+                        st, cases, tile_case, ntiles, k, duty);
 }
 
 cudaError_t launch_lattice_batch_f32(const BatchLattice<float>* cases, const int* tile_case, int ntiles, int k,
@@ -117,17 +119,15 @@ cudaError_t launch_ellipse_batch(const BatchParticles* cases, const BatchEllipse
                                  cudaStream_t st) {
   if (ell.n == 0) return cudaSuccess;
   const int blocks = (ell.rows + ELL_WARPS - 1) / ELL_WARPS;
-  particle_ellipse_batch_kernel<<<(unsigned)(blocks * ell.n), 32 * ELL_WARPS, 0, st>>>(cases, ell.items, blocks, k,
-                                                                                      kdev);
-  return cudaGetLastError();
+  return launch_chained(particle_ellipse_batch_kernel, dim3((unsigned)(blocks * ell.n)), dim3(32 * ELL_WARPS), st, cases,
+                        ell.items, blocks, k, kdev);
 }
 cudaError_t launch_particle_step_batch(const BatchParticles* cases, const int2* items, int nitems, int k,
                                        const BatchEllipses& ell, cudaStream_t st) {
   if (nitems == 0) return cudaSuccess;
   const int group = step_group_size(nitems);
-  particle_step_batch_kernel<<<(unsigned)((nitems + group - 1) / group), STEP_THREADS, 0, st>>>(cases, items, nitems, k,
-                                                                                               group);
-  const cudaError_t e = cudaGetLastError();
+  const cudaError_t e = launch_chained(particle_step_batch_kernel, dim3((unsigned)((nitems + group - 1) / group)),
+                                       dim3(STEP_THREADS), st, cases, items, nitems, k, group);
   return e != cudaSuccess ? e : launch_ellipse_batch(cases, ell, k, nullptr, st);
 }
 

@@ -105,6 +105,16 @@ struct TileLists {
   int* next_count;  // counts of the other list buffer, cleared by the lattice kernel (may be null)
 };
 
+// Start of a kernel that launch_chained puts into a stream: it may become
+// resident while the kernel before it drains, and waits here until that kernel
+// has completed and its writes are visible; then the next one may come in.
+__device__ __forceinline__ void begin_chained() {
+#ifdef __CUDA_ARCH__
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+#endif
+}
+
 // Contact decision d_ij^2 < (R_i + R_j + zeta)^2 in FP64 without contraction,
 // so that every device and the reference arithmetic take it identically.
 __device__ __forceinline__ bool in_contact_range(double xi, double yi, double ri, double xj, double yj,

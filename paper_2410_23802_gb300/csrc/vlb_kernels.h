@@ -5,6 +5,22 @@
 
 namespace vlb {
 
+// Launch of a kernel that begins with begin_chained(): behind another kernel
+// of the stream its CTAs are brought in before that one has drained.
+template <class... P, class... A>
+cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t st, A... args) {
+  cudaLaunchAttribute early{};
+  early.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  early.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.stream = st;
+  cfg.attrs = &early;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
 // Constants of the particle kernels (Sec. 2.3 and the contact model).
 struct ParticleConst {
   int np, nx, ny, per_x, per_y, ntx, nty;

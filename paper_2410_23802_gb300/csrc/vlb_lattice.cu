@@ -16,6 +16,7 @@ __global__ void __launch_bounds__(32 * tile_warps<C>(), sizeof(C) == 4 ? VLB_LAT
 lattice_kernel(const LatticeConst<C> K, const StepBuffers B, const ParticleArrays P, const TileLists TL, int duty) {
   constexpr int WARPS = tile_warps<C>();
   __shared__ PartTile<C> list[WARPS][TILE_CAP];
+  begin_chained();
   const int lane = threadIdx.x, warp = threadIdx.y;
   if (blockIdx.y < duty) {
     const int ntiles = K.ntx * K.nty, span = duty_span(ntiles);
@@ -124,13 +125,11 @@ static cudaError_t launch_mode(int mode, const LatticeConst<C>& K, const StepBuf
   const int duty_ctas = (ntiles + per_cta - 1) / per_cta;
   const int duty = mode != MODE_MACROS && K.np > 0 ? (duty_ctas + across - 1) / across : 0;
   const dim3 grid(across, K.nty + duty), block(32, WARPS);
+  auto go = [&](auto kernel) { return launch_chained(kernel, grid, block, st, K, B, P, TL, duty); };
   // kernels with the held-temperature path only where some particle is held
-  if (mode == MODE_INIT) lattice_kernel<S, C, MODE_INIT, false><<<grid, block, 0, st>>>(K, B, P, TL, duty);
-  else if (mode == MODE_STEP && K.any_held) lattice_kernel<S, C, MODE_STEP, true><<<grid, block, 0, st>>>(K, B, P, TL, duty);
-  else if (mode == MODE_STEP) lattice_kernel<S, C, MODE_STEP, false><<<grid, block, 0, st>>>(K, B, P, TL, duty);
-  else if (K.any_held) lattice_kernel<S, C, MODE_MACROS, true><<<grid, block, 0, st>>>(K, B, P, TL, duty);
-  else lattice_kernel<S, C, MODE_MACROS, false><<<grid, block, 0, st>>>(K, B, P, TL, duty);
-  return cudaGetLastError();
+  if (mode == MODE_INIT) return go(lattice_kernel<S, C, MODE_INIT, false>);
+  if (mode == MODE_STEP) return K.any_held ? go(lattice_kernel<S, C, MODE_STEP, true>) : go(lattice_kernel<S, C, MODE_STEP, false>);
+  return K.any_held ? go(lattice_kernel<S, C, MODE_MACROS, true>) : go(lattice_kernel<S, C, MODE_MACROS, false>);
 }
 
 cudaError_t launch_lattice_f32(int mode, const LatticeConst<float>& K, const StepBuffers& B,

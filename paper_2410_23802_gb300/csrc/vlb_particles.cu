@@ -26,6 +26,7 @@ __global__ void __launch_bounds__(32 * BAND_WARPS) particle_band_kernel(const Pa
 __global__ void __launch_bounds__(32 * ELL_WARPS)
     particle_ellipse_kernel(const ParticleConst c, const ParticleArrays P, const int* __restrict__ ell, int blocks) {
   __shared__ int s_queue[ELL_WARPS][32];
+  begin_chained();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int i = blockIdx.x / blocks, by = (blockIdx.x - i * blocks) * ELL_WARPS + warp;
   if (by >= 2 * c.band_off + 1) return;  // the whole warp
@@ -40,6 +41,7 @@ __global__ void __launch_bounds__(STEP_THREADS) particle_step_kernel(const __gri
                                                                      const __grid_constant__ TileLists TL,
                                                                      unsigned* err, int group) {
   __shared__ StepShared sh;
+  begin_chained();
   const int p0 = blockIdx.x * group;
   step_group(min(group, c.np - p0), [&](int s) { return StepRef{&c, &P, &TL, err, p0 + s, c.band_stamp}; }, sh);
 }
@@ -56,22 +58,26 @@ static cudaError_t launch_ellipses(const ParticleConst& c, const ParticleArrays&
                                    cudaStream_t st) {
   if (nell > 0) {
     const int blocks = (2 * c.band_off + ELL_WARPS) / ELL_WARPS;  // rows 0 .. 2 band_off
-    particle_ellipse_kernel<<<(unsigned)(blocks * nell), 32 * ELL_WARPS, 0, st>>>(c, P, ell, blocks);
+    return launch_chained(particle_ellipse_kernel, dim3((unsigned)(blocks * nell)), dim3(32 * ELL_WARPS), st, c, P, ell,
+                          blocks);
   }
-  return cudaGetLastError();
+  return cudaSuccess;
 }
 cudaError_t launch_particle_band(const ParticleConst& c, const ParticleArrays& P, const TileLists& TL, const int* ell,
                                  int nell, unsigned* err, cudaStream_t st) {
   if (c.np == 0) return cudaSuccess;
   const unsigned grid = (unsigned)((c.np + BAND_WARPS - 1) / BAND_WARPS);
   particle_band_kernel<<<grid, 32 * BAND_WARPS, 0, st>>>(c, P, TL, err);
+  if (const cudaError_t e = cudaGetLastError(); e != cudaSuccess) return e;
   return launch_ellipses(c, P, ell, nell, st);
 }
 cudaError_t launch_particle_step(const ParticleConst& c, const ParticleArrays& P, const TileLists& TL, const int* ell,
                                  int nell, unsigned* err, cudaStream_t st) {
   if (c.np == 0) return cudaSuccess;
   const int group = step_group_size(c.np);
-  particle_step_kernel<<<(unsigned)((c.np + group - 1) / group), STEP_THREADS, 0, st>>>(c, P, TL, err, group);
+  const cudaError_t e = launch_chained(particle_step_kernel, dim3((unsigned)((c.np + group - 1) / group)),
+                                       dim3(STEP_THREADS), st, c, P, TL, err, group);
+  if (e != cudaSuccess) return e;
   return launch_ellipses(c, P, ell, nell, st);
 }
 }  // namespace vlb
