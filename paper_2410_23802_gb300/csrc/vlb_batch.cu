@@ -44,7 +44,7 @@ lattice_batch_kernel(const BatchLattice<C>* __restrict__ cases, const int* __res
     }
     return;
   }
-  const int block = blockIdx.x - duty, tile = block / PARTS;
+  const int block = blockIdx.x - duty, tile = block / PARTS, part = WARPS == 1 ? block % PARTS : warp;
   {
     const int* src = reinterpret_cast<const int*>(cases + tile_case[tile]);
     int* dst = reinterpret_cast<int*>(&d);
@@ -54,7 +54,7 @@ lattice_batch_kernel(const BatchLattice<C>* __restrict__ cases, const int* __res
   const StepBuffers& B = d.B[d.cur ^ par];
   const int t = tile - d.tile0;
   const int tile_y = t / d.K.ntx, tile_x = t - tile_y * d.K.ntx;
-  const CellAt at = cell_at<S>(tile_x, tile_y, WARPS == 1 ? block % PARTS : warp, lane);
+  const CellAt at = cell_at<S>(tile_x, tile_y, part, lane);
   if (WARPS == 1 && tile_x * TILE_X + at.bx >= d.K.nx) return;  // a strip beyond the lattice
   const ListHead head = list_head(d.TL[1 - (d.tl ^ par)], t, lane);
   Pair<C> p[9];
