@@ -530,7 +530,9 @@ __device__ __forceinline__ void step_group(int n, const Ref& ref, StepShared& sh
 
 // Particles per CTA of the particle step: one while every particle can have a
 // CTA to itself (four of them are resident per SM, 608 on 152 SMs), then as
-// many as keep the grid at that size, up to STEP_GROUP.
+// many as keep the grid at that size, up to STEP_GROUP (2048 disks, us per
+// step of the 2048^2 cavity: at most 304 CTAs 117.4, 456 115.7, 608 114.7,
+// 1216 117.2).
 inline int step_group_size(int n) {
   const int g = (n + 607) / 608;
   return g < 1 ? 1 : (g > STEP_GROUP ? STEP_GROUP : g);
