@@ -781,8 +781,8 @@ vlb_status vlb_step(vlb_handle* h, int32_t nsteps) {
 
 // Descriptors of one batch call, packed into one host block and one device
 // copy: the particle descriptors, the (case, particle) items, and per group
-// of handles that share a lattice kernel (precision, storage, held path) the
-// lattice descriptors and the tile-to-case table.
+// of handles that share a lattice launch (precision, held path; storage too in
+// the persistent form) the lattice descriptors and the tile-to-case table.
 namespace {
 struct BatchGroup {
   bool f64 = false, held = false;
@@ -845,6 +845,7 @@ void fill_lattice_desc(vlb_handle* h, const LatticeConst<C>& K, int tile0, Batch
   d.cur = h->cur;
   d.tl = h->tl;
   d.stamp = h->PC.band_stamp;
+  d.storage = h->storage;
 }
 }  // namespace
 
@@ -902,7 +903,7 @@ static vlb_status step_batch_impl(vlb_handle* const* hs, int32_t n, int32_t nste
     const int storage = f64 ? 0 : h->storage;
     BatchGroup* g = nullptr;
     for (auto& q : groups)
-      if (q.f64 == f64 && q.held == held && q.storage == storage) g = &q;
+      if (q.f64 == f64 && q.held == held && (!persistent || q.storage == storage)) g = &q;
     if (!g) {
       groups.emplace_back();
       g = &groups.back();
@@ -910,6 +911,7 @@ static vlb_status step_batch_impl(vlb_handle* const* hs, int32_t n, int32_t nste
       g->held = held;
       g->storage = storage;
     }
+    if (g->storage != storage) g->storage = STORE_ANY;
     g->handles.push_back(i);
     for (int k = 0; k < h->np; ++k) items.push_back(make_int2(i, k));
     if (h->nell > 0) {

@@ -47,6 +47,7 @@ struct BatchLattice {
   ParticleArrays P;
   int tile0;         // first tile of the case in the batched grid (tiles row by row)
   int cur, tl, stamp;
+  int storage;       // STORE_* of the case
 };
 struct BatchParticles {
   ParticleConst c;
@@ -57,7 +58,7 @@ struct BatchParticles {
 };
 
 // Storage of the populations of the FP32-arithmetic kernels.
-enum : int { STORE_F32 = 0, STORE_F16 = 1, STORE_BF16 = 2 };
+enum : int { STORE_F32 = 0, STORE_F16 = 1, STORE_BF16 = 2, STORE_ANY = 3 };  // ANY: several in one launch
 
 cudaError_t launch_lattice_f32(int mode, const LatticeConst<float>& K, const StepBuffers& B,
                                const ParticleArrays& P, const TileLists& TL, cudaStream_t st, int storage);
@@ -92,7 +93,7 @@ cudaError_t launch_particle_step_batch(const BatchParticles* cases, const int2* 
 
 // Batched step k: lattice tiles map to their case through tile_case.
 // `held`: the held-temperature path (every case of the launch shares
-// precision, storage and held).
+// arithmetic, held, and the storage unless that is STORE_ANY).
 cudaError_t launch_lattice_batch_f32(const BatchLattice<float>* cases, const int* tile_case, int ntiles, int k,
                                      int storage, bool held, cudaStream_t st);
 cudaError_t launch_lattice_batch_f64(const BatchLattice<double>* cases, const int* tile_case, int ntiles, int k,
