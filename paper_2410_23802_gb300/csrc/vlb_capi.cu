@@ -1511,9 +1511,10 @@ static cudaError_t copy_populations(vlb_handle* h, int b, char* out, const char*
   cudaError_t e = cudaMalloc(reinterpret_cast<void**>(&scratch), 2 * plane);
   if (e == cudaErrorMemoryAllocation) {
     cudaGetLastError();
-    std::vector<char> pairs(2 * plane), two(2 * plane);
+    std::unique_ptr<char[]> pairs(new (std::nothrow) char[2 * plane]), two(new (std::nothrow) char[2 * plane]);
+    if (!pairs || !two) return e;
     auto split = [&](bool join) {
-      char *q = pairs.data(), *f = two.data(), *g = f + plane;
+      char *q = pairs.get(), *f = two.get(), *g = f + plane;
       if (h->ssize == 8) split_on_host((uint64_t*)q, (uint64_t*)f, (uint64_t*)g, n, join);
       else if (h->ssize == 4) split_on_host((uint32_t*)q, (uint32_t*)f, (uint32_t*)g, n, join);
       else split_on_host((uint16_t*)q, (uint16_t*)f, (uint16_t*)g, n, join);
@@ -1522,13 +1523,13 @@ static cudaError_t copy_populations(vlb_handle* h, int b, char* out, const char*
     for (int i = 0; i < 9 && e == cudaSuccess; ++i) {
       char* dev = static_cast<char*>(h->pop[b]) + 2 * plane * i;
       if (in) {
-        for (int q = 0; q < 2; ++q) std::memcpy(two.data() + q * plane, in + (9 * q + i) * plane, plane);
+        for (int q = 0; q < 2; ++q) std::memcpy(two.get() + q * plane, in + (9 * q + i) * plane, plane);
         split(true);
-        e = cudaMemcpy(dev, pairs.data(), 2 * plane, cudaMemcpyHostToDevice);
+        e = cudaMemcpy(dev, pairs.get(), 2 * plane, cudaMemcpyHostToDevice);
       } else {
-        e = cudaMemcpy(pairs.data(), dev, 2 * plane, cudaMemcpyDeviceToHost);
+        e = cudaMemcpy(pairs.get(), dev, 2 * plane, cudaMemcpyDeviceToHost);
         split(false);
-        for (int q = 0; q < 2; ++q) std::memcpy(out + (9 * q + i) * plane, two.data() + q * plane, plane);
+        for (int q = 0; q < 2; ++q) std::memcpy(out + (9 * q + i) * plane, two.get() + q * plane, plane);
       }
     }
     return e;
