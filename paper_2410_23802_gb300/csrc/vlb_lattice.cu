@@ -11,6 +11,18 @@ namespace vlb {
 // full: on a 100 x 400 channel, tiles of four warps put three CTAs on some SMs
 // and two on others and gave the fourth tile column 4 live lanes in 32.
 // The first `duty` rows of the grid have the once-per-tile work (tile_duties).
+//
+// What bounds it (GB300, one launch per step, FP32 at 152 B per cell update):
+//   FP32, 2048^2 with 2048 disks: memory and the particle tiles' chain of list,
+//     record and band table; 110.3 us = 5.78 TB/s (127 us before: a list per
+//     CTA behind a barrier, exchange sums over shared memory, f and g in planes
+//     of their own, both collisions by the full moment matrices).  Without
+//     particles 96 us = 6.6 TB/s.
+//   16-bit storage, same case: instruction issue, 527 per warp of 32 cells
+//     (880 before); FP16 92 us, BF16 91 us.
+//   FP64, 100 x 400: the FP64 pipe (67 % busy); 37 us (56 before).
+//   A lattice of less than a wave of warps (100 x 400 FP32): the latency of one
+//     cell, 3.7 us.
 template <class S, class C, int MODE, bool HOLD>
 __global__ void __launch_bounds__(32 * tile_warps<C>(), sizeof(C) == 4 ? VLB_LATTICE_MIN_BLOCKS : 1)
 lattice_kernel(const LatticeConst<C> K, const StepBuffers B, const ParticleArrays P, const TileLists TL, int duty) {
