@@ -6,7 +6,7 @@
 // tiles (form 1).
 #include <atomic>
 
-#include "vlb_lattice_body.cuh"
+#include "vlb_lattice_held.cuh"
 #include "vlb_particle_body.cuh"
 
 namespace vlb {
@@ -21,10 +21,7 @@ __device__ __forceinline__ void batch_tile(const BatchLattice<C>& d, int t, int 
   const CellAt at = cell_at<S>(tile_x, tile_y, part, lane);
   if (tile_warps<C>() == 1 && tile_x * TILE_X + at.bx >= d.K.nx) return;  // a strip beyond the lattice
   const ListHead head = list_head(d.TL[1 - (d.tl ^ par)], t, lane);
-  Pair<C> p[9];
-  C s_old;
-  pull_direct<S, C, MODE_STEP>(d.K, B, at, p, s_old);
-  cell_body<S, C, MODE_STEP, HOLD>(d.K, B, d.P, at, head, p, s_old, list, band_stamp_after(d.stamp, k + 1));
+  lattice_cell<S, C, MODE_STEP, HOLD>(d.K, B, d.P, at, head, list, band_stamp_after(d.stamp, k + 1));
 }
 // Storage of a launch whose cases do not share one: each tile takes the code
 // of its case's.  A round of served cases of both kinds then takes one launch
@@ -85,14 +82,16 @@ lattice_batch_kernel(const BatchLattice<C>* __restrict__ cases, const int* __res
 }
 
 // The same over the particles of many cases, step k of a batch call; `group`
-// (case, particle) items per CTA (see step_group).
+// (case, particle) items per CTA (see step_group).  HELD: some case of the
+// batch has held particles.
+template <bool HELD>
 __global__ void __launch_bounds__(STEP_THREADS)
     particle_step_batch_kernel(const BatchParticles* __restrict__ cases, const int2* __restrict__ items, int nitems,
                                int k, int group) {
   __shared__ StepShared sh;
   begin_chained();
   const int i0 = blockIdx.x * group;
-  step_group(min(group, nitems - i0), [&](int s) {
+  step_group<HELD>(min(group, nitems - i0), [&](int s) {
     const int2 it = items[i0 + s];
     const BatchParticles& d = cases[it.x];
     return StepRef{&d.c, &d.P, &d.TL[1 - (d.tl ^ (k & 1))], d.err, it.y, band_stamp_after(d.stamp, k + 1)};
@@ -116,12 +115,13 @@ __global__ void __launch_bounds__(32 * ELL_WARPS)
 template <class S, class C>
 static cudaError_t launch_batch(const BatchLattice<C>* cases, const int* tile_case, int ntiles, int k, bool held,
                                 cudaStream_t st) {
+  constexpr bool HOLD = !std::is_same<S, AnyStorage>::value;  // (held lattices of one launch share their storage)
   if (ntiles == 0) return cudaSuccess;
   constexpr int WARPS = tile_warps<C>();
   const dim3 block(32, WARPS);
   const int per_cta = duty_span(ntiles) * WARPS, duty = (ntiles + per_cta - 1) / per_cta;
   const unsigned grid = (unsigned)duty + (unsigned)ntiles * (TILE_Y / WARPS);
-  return launch_chained(held ? lattice_batch_kernel<S, C, true> : lattice_batch_kernel<S, C, false>, dim3(grid), block,
+  return launch_chained(held ? lattice_batch_kernel<S, C, HOLD> : lattice_batch_kernel<S, C, false>, dim3(grid), block,
                         st, cases, tile_case, ntiles, k, duty);
 }
 
@@ -147,12 +147,12 @@ cudaError_t launch_ellipse_batch(const BatchParticles* cases, const BatchEllipse
   particle_ellipse_batch_kernel<<<grid, block, 0, st>>>(cases, ell.items, blocks, k, kdev);
   return cudaGetLastError();
 }
-cudaError_t launch_particle_step_batch(const BatchParticles* cases, const int2* items, int nitems, int k,
+cudaError_t launch_particle_step_batch(const BatchParticles* cases, const int2* items, int nitems, int k, bool held,
                                        const BatchEllipses& ell, cudaStream_t st) {
   if (nitems == 0) return cudaSuccess;
   const int group = step_group_size(nitems);
-  const cudaError_t e = launch_chained(particle_step_batch_kernel, dim3((unsigned)((nitems + group - 1) / group)),
-                                       dim3(STEP_THREADS), st, cases, items, nitems, k, group);
+  const cudaError_t e = launch_chained(held ? particle_step_batch_kernel<true> : particle_step_batch_kernel<false>,
+                                       dim3((unsigned)((nitems + group - 1) / group)), dim3(STEP_THREADS), st, cases, items, nitems, k, group);
   return e != cudaSuccess ? e : launch_ellipse_batch(cases, ell, k, nullptr, st);
 }
 
@@ -190,7 +190,7 @@ __device__ bool wait_count(const int* count, int target, long long limit_ns) {
 // level kn, after the last tile of its case (whose exchange sums, contact
 // partners and cleared list buffer it reads).  Inlined: as a call it cost
 // the tile path more (spills around the call) than its own FP64 code does.
-template <class C>
+template <class C, bool HOLD>
 __device__ __forceinline__ void persistent_particle(const PersistentBatch<C>& A, int i, int kn, int* queue) {
   const int lane = threadIdx.x & 31;
   if (i >= A.npitems) return;
@@ -210,7 +210,7 @@ __device__ __forceinline__ void persistent_particle(const PersistentBatch<C>& A,
   record_constants(pd.P, it.y, u.R, u.Rb, rq);
   update_velocity(pd.c, pd.P, it.y, lane, lane < 4, u, rq, pd.err);
   __syncwarp();  // the record and tile range are visible to every lane
-  band_one(pd.c, pd.P, pd.TL[1 - (pd.tl ^ (kn & 1))], pd.err, it.y, band_stamp_after(pd.stamp, kn + 1), queue, lane);
+  band_one<HOLD>(pd.c, pd.P, pd.TL[1 - (pd.tl ^ (kn & 1))], pd.err, it.y, band_stamp_after(pd.stamp, kn + 1), queue, lane);
 }
 
 // Tiles per work chunk of the persistent launch: a CTA takes the next chunk
@@ -284,11 +284,7 @@ lattice_persistent_kernel(const __grid_constant__ PersistentBatch<C> A) {
       const int lane = threadIdx.x, warp = threadIdx.y;
       const CellAt at = cell_at<S>(tile_x, tile_y, warp, lane);
       const ListHead head = list_head(TL, lt, lane);
-      Pair<C> p[9];
-      C s_old;
-      pull_direct<S, C, MODE_STEP>(d.K, B, at, p, s_old);
-      cell_body<S, C, MODE_STEP, HOLD>(d.K, B, d.P, at, head, p, s_old, sh.list[warp],
-                                       band_stamp_after(d.stamp, s_k + 1));
+      lattice_cell<S, C, MODE_STEP, HOLD>(d.K, B, d.P, at, head, sh.list[warp], band_stamp_after(d.stamp, s_k + 1));
       if (warp == 0) {
         if (lane == 0) TL.next_count[lt] = 0;  // the next particle step fills the other list buffer
         if (head.count > 1) contact_pairs(d.K, d.P, TL.ids, head.count, lt, lane, B.err);
@@ -304,7 +300,7 @@ lattice_persistent_kernel(const __grid_constant__ PersistentBatch<C> A) {
         ++s_pend;
       }
     } else {
-      persistent_particle<C>(A, (item - A.ntiles) * NWARPS + (tid >> 5), s_k + 1, sh.queue[tid >> 5]);
+      persistent_particle<C, HOLD>(A, (item - A.ntiles) * NWARPS + (tid >> 5), s_k + 1, sh.queue[tid >> 5]);
       __syncthreads();  // the band queues are free
     }
     if (item + 1 < end) {  // the next tile of this chunk (every thread knows it)

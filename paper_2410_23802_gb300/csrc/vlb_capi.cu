@@ -192,6 +192,7 @@ static void fill_const(vlb_handle* h, LatticeConst<C>& K) {
   // Eq. 5 with the rules of Sec. 3
   const double sp = 1.0 / p.tau_f;
   const double sq = 1.0 / (0.5 + p.lambda_q_flow / (p.tau_f - 0.5));
+  K.s_e = C(p.s_e); K.s_eps = C(p.s_e); K.s_q = C(sq); K.s_p = C(sp);
   K.q_e = C(p.s_e / 4.0); K.q_q = C(sq / 12.0); K.q_p = C(sp / 4.0);
   K.q_fu = C((1.0 - 0.5 * p.s_e) / 6.0); K.q_f4 = C(-(1.0 - 0.5 * sq) / 12.0); K.q_f7 = C(0.5 * (1.0 - 0.5 * sp));
   // Eqs. 11, 22 with rho_f = c_vf = 1; lambda_f = nu / Pr
@@ -658,7 +659,7 @@ static vlb_status initialize(vlb_handle* h) {
   h->K32.band_off = h->K64.band_off = band_off;
   int any_held = 0;
   for (int v : h->hfix) any_held |= v;
-  h->K32.any_held = h->K64.any_held = any_held;
+  h->K32.any_held = h->K64.any_held = h->PC.any_held = any_held;
   c.rho_ratio = p.rho_ratio; c.gx = p.gravity[0]; c.gy = p.gravity[1];
   c.zeta = p.contact_range; c.eps_p = p.contact_eps_p; c.eps_w = p.contact_eps_w;
   c.contact_scale = std::fabs(p.rho_ratio - 1.0) * std::hypot(p.gravity[0], p.gravity[1]) * M_PI;
@@ -782,7 +783,8 @@ vlb_status vlb_step(vlb_handle* h, int32_t nsteps) {
 // Descriptors of one batch call, packed into one host block and one device
 // copy: the particle descriptors, the (case, particle) items, and per group
 // of handles that share a lattice launch (precision, held path; storage too in
-// the persistent form) the lattice descriptors and the tile-to-case table.
+// the persistent form and with held particles, see vlb_lattice_held.cuh) the
+// lattice descriptors and the tile-to-case table.
 namespace {
 struct BatchGroup {
   bool f64 = false, held = false;
@@ -896,14 +898,16 @@ static vlb_status step_batch_impl(vlb_handle* const* hs, int32_t n, int32_t nste
   std::vector<BatchGroup> groups;
   std::vector<int2> items, eitems;
   int erows = 0;
+  bool any_held = false;
   for (int i = 0; i < n; ++i) {
     vlb_handle* h = hs[i];
     const bool f64 = h->p.precision == VLB_FP64;
     const bool held = f64 ? h->K64.any_held : h->K32.any_held;
+    any_held |= held;
     const int storage = f64 ? 0 : h->storage;
     BatchGroup* g = nullptr;
     for (auto& q : groups)
-      if (q.f64 == f64 && q.held == held && (!persistent || q.storage == storage)) g = &q;
+      if (q.f64 == f64 && q.held == held && ((!persistent && !held) || q.storage == storage)) g = &q;
     if (!g) {
       groups.emplace_back();
       g = &groups.back();
@@ -1019,7 +1023,7 @@ static vlb_status step_batch_impl(vlb_handle* const* hs, int32_t n, int32_t nste
   const BatchEllipses ell{reinterpret_cast<const int2*>(dev + eitems_off), (int)eitems.size(), erows};
   if (!persistent) {
     for (int k = 0; k < nsteps && e == cudaSuccess; ++k) {
-      e = launch_particle_step_batch(d_part, d_items, nitems, k, ell, bs);
+      e = launch_particle_step_batch(d_part, d_items, nitems, k, any_held, ell, bs);
       for (auto& g : groups) {
         if (e != cudaSuccess) break;
         const int* table = reinterpret_cast<const int*>(dev + g.table_off);
@@ -1055,7 +1059,7 @@ static vlb_status step_batch_impl(vlb_handle* const* hs, int32_t n, int32_t nste
         return launch_ellipse_batch(d_part, ell, 0, &reinterpret_cast<const BatchCtl*>(dev + groups[0].ctl_off)->k, bs);
       return cudaSuccess;
     };
-    e = launch_particle_step_batch(d_part, d_items, nitems, 0, ell, bs);
+    e = launch_particle_step_batch(d_part, d_items, nitems, 0, any_held, ell, bs);
     // the steps' launches are the same every step (the step index lives on
     // the device): up to kGraphSteps of them are captured into one CUDA graph,
     // replayed as often as it fits, and the rest launched plainly
@@ -1633,7 +1637,7 @@ vlb_status vlb_load_state(vlb_handle* h, const void* buf, uint64_t bytes) {
   }
   int any_held = 0;
   for (int v : h->hfix) any_held |= v;
-  h->K32.any_held = h->K64.any_held = any_held;
+  h->K32.any_held = h->K64.any_held = h->PC.any_held = any_held;
   if ((s = upload_ellipses(h)) != VLB_OK) return s;
   h->cur = I.cur;
   h->tl = I.tl;

@@ -178,6 +178,7 @@ struct LatticeConst {
   // s_eps: s_e / 4, s_q / 12, s_p / 4, and the forcing's (1 - s_e / 2) / 6,
   // -(1 - s_q / 2) / 12, (1 - s_p / 2) / 2
   C q_e, q_q, q_p, q_fu, q_f4, q_f7;
+  C s_e, s_eps, s_q, s_p;  // the rates themselves (lattices with held particles)
   // thermal (Eqs. 11, 18-22)
   C cv_f, cv_s, cref, lam_f, rates_mode;
   C bx, by, T_ref, T_fluid;  // buoyancy b = -rho_f beta g; T_f = initial fluid temperature

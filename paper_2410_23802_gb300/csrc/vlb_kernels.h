@@ -27,6 +27,7 @@ struct ParticleConst {
   int outflow[4];    // open sides (no wall contact there)
   int band_off;      // half-width of the band tables (cells)
   int band_stamp;    // level stamp written into the band tables
+  int any_held;      // some particle is held: areas as vlb_raster_held.cuh has them
   double rho_ratio, gx, gy;
   double zeta, eps_p, eps_w, contact_scale;  // scale = |rho_r - 1| rho_f |g| pi
   double margin;                             // tile-range margin around each disk (cells)
@@ -88,12 +89,13 @@ struct BatchEllipses {
   const int2* items;
   int n, rows;
 };
-cudaError_t launch_particle_step_batch(const BatchParticles* cases, const int2* items, int nitems, int k,
+// (held: some case of the batch has held particles)
+cudaError_t launch_particle_step_batch(const BatchParticles* cases, const int2* items, int nitems, int k, bool held,
                                        const BatchEllipses& ell, cudaStream_t st);
 
 // Batched step k: lattice tiles map to their case through tile_case.
 // `held`: the held-temperature path (every case of the launch shares
-// arithmetic, held, and the storage unless that is STORE_ANY).
+// arithmetic, held, and the storage unless that is STORE_ANY, never with held).
 cudaError_t launch_lattice_batch_f32(const BatchLattice<float>* cases, const int* tile_case, int ntiles, int k,
                                      int storage, bool held, cudaStream_t st);
 cudaError_t launch_lattice_batch_f64(const BatchLattice<double>* cases, const int* tile_case, int ntiles, int k,

@@ -1,6 +1,6 @@
 // The single-case lattice kernels: the fused step (see vlb_lattice_body.cuh),
 // the ownership dump and the FP64 audits.
-#include "vlb_lattice_body.cuh"
+#include "vlb_lattice_held.cuh"
 
 namespace vlb {
 
@@ -39,10 +39,7 @@ lattice_kernel(const LatticeConst<C> K, const StepBuffers B, const ParticleArray
   const CellAt at = cell_at<S>(tile_x, tile_y, WARPS == 1 ? blockIdx.x % TILE_Y : warp, lane);
   if (WARPS == 1 && tile_x * TILE_X + at.bx >= K.nx) return;  // a strip beyond the lattice
   const ListHead head = list_head(TL, tile_y * K.ntx + tile_x, lane);
-  Pair<C> p[9];
-  C s_old;
-  pull_direct<S, C, MODE>(K, B, at, p, s_old);
-  cell_body<S, C, MODE, HOLD>(K, B, P, at, head, p, s_old, list[warp], K.band_stamp);
+  lattice_cell<S, C, MODE, HOLD>(K, B, P, at, head, list[warp], K.band_stamp);
 }
 
 // Ownership of every cell at the current level, from the same raster code as
@@ -139,7 +136,10 @@ static cudaError_t launch_mode(int mode, const LatticeConst<C>& K, const StepBuf
   const dim3 grid(across, K.nty + duty), block(32, WARPS);
   auto go = [&](auto kernel) { return launch_chained(kernel, grid, block, st, K, B, P, TL, duty); };
   // kernels with the held-temperature path only where some particle is held
-  if (mode == MODE_INIT) return go(lattice_kernel<S, C, MODE_INIT, false>);
+  // (FP64 holds nothing at the initial state, which is an equilibrium)
+  if (mode == MODE_INIT)
+    return sizeof(C) == 4 && K.any_held ? go(lattice_kernel<S, C, MODE_INIT, sizeof(C) == 4>)
+                                        : go(lattice_kernel<S, C, MODE_INIT, false>);
   if (mode == MODE_STEP) return K.any_held ? go(lattice_kernel<S, C, MODE_STEP, true>) : go(lattice_kernel<S, C, MODE_STEP, false>);
   return K.any_held ? go(lattice_kernel<S, C, MODE_MACROS, true>) : go(lattice_kernel<S, C, MODE_MACROS, false>);
 }

@@ -22,6 +22,7 @@
 #include "vlb_common.cuh"
 #include "vlb_kernels.h"
 #include "vlb_raster.cuh"
+#include "vlb_raster_held.cuh"
 
 namespace vlb {
 
@@ -279,11 +280,15 @@ __device__ __forceinline__ bool in_band(const RasterRec& rc, int x, int y) {
   tile_coordinate(rc.yi - (y - ty), rc.yfh, rc.yfl, yh, yl);
   return quick_class_at(tx, ty, xh, xl, yh, yl, rc.far2, rc.near2) == CELL_BAND;
 }
-// Entry (bx, by) of a particle's table.
+// Entry (bx, by) of a particle's table.  HELD: compiled with the areas of
+// lattices with held particles, taken where `held` says so (in the kernels of
+// all other lattices they would cost registers).
+template <bool HELD>
 __device__ __forceinline__ void band_fill(const RasterRec& rc, int2* table, int off, int stamp, float i2R, int bx,
-                                          int by) {
+                                          int by, int held) {
   float f;
-  const int cls = disk_band_cell(rc, bx - off, by - off, i2R, f);
+  const int cls = HELD && held ? held_band_cell(rc, rc.xi - off + bx, rc.yi - off + by, f)
+                               : disk_band_cell(rc, bx - off, by - off, i2R, f);
   table[(long long)by * (2 * off + 1) + bx] = make_int2(cls | (stamp << 2), __float_as_int(f));
 }
 __device__ __forceinline__ int2* band_table(const ParticleArrays& P, int off, int p) {
@@ -308,6 +313,7 @@ __device__ __forceinline__ void append_to_tiles(const TileLists& TL, int ntx, in
 // particle steps inside a persistent launch.
 constexpr int BAND_WARPS = 4;    // particles per CTA
 constexpr int BAND_QUEUE = 256;  // queued band cells per warp before an evaluation pass
+template <bool HELD>
 __device__ __forceinline__ void band_one(const ParticleConst& c, const ParticleArrays& P, const TileLists& TL,
                                          unsigned* err, int p, int stamp, int* queue, int lane) {
   const RasterRec rc = P.rec[p];
@@ -318,7 +324,7 @@ __device__ __forceinline__ void band_one(const ParticleConst& c, const ParticleA
   const float i2R = 0.5f / rc.r;
   auto evaluate = [&](int nq) {
     __syncwarp();
-    for (int j = lane; j < nq; j += 32) band_fill(rc, table, off, stamp, i2R, queue[j] % bw, queue[j] / bw);
+    for (int j = lane; j < nq; j += 32) band_fill<HELD>(rc, table, off, stamp, i2R, queue[j] % bw, queue[j] / bw, c.any_held);
     __syncwarp();
   };
   int nq = 0;
@@ -377,7 +383,7 @@ struct StepSlot {
   int2* table;
   int4 rg;
   float i2R;
-  int nx, ny, off, stamp, row0;  // row0: rows of the slots before
+  int nx, ny, off, stamp, held, row0;  // row0: rows of the slots before
 };
 struct StepShared {
   StepSlot slot[STEP_GROUP];
@@ -392,6 +398,7 @@ struct StepShared {
 __device__ __forceinline__ void band_barrier() { asm volatile("bar.sync 1, %0;" ::"n"(STEP_BAND) : "memory"); }
 
 // The band tables of the CTA's slots (t: 0 .. STEP_BAND - 1).
+template <bool HELD>
 __device__ __forceinline__ void band_group(StepShared& sh, int n, int t) {
   const int lane = t & 31, warp = t >> 5;
   const int rows = sh.rows;
@@ -468,14 +475,14 @@ __device__ __forceinline__ void band_group(StepShared& sh, int n, int t) {
         if (!mine[g]) continue;
         const int s = e[g].x >> 20, bx = e[g].x & 0xfffff, by = e[g].y;
         const StepSlot& S = sh.slot[s];
-        band_fill(S.rc, S.table, S.off, S.stamp, S.i2R, bx, by);
+        band_fill<HELD>(S.rc, S.table, S.off, S.stamp, S.i2R, bx, by, S.held);
       }
     }
   }
 }
 
 // The particle step of the n <= STEP_GROUP particles ref(0) .. ref(n - 1).
-template <class Ref>
+template <bool HELD, class Ref>
 __device__ __forceinline__ void step_group(int n, const Ref& ref, StepShared& sh) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   UpdateLane u;
@@ -500,6 +507,7 @@ __device__ __forceinline__ void step_group(int n, const Ref& ref, StepShared& sh
       const double R = r.P->r[r.p], Rb = r.P->rb[r.p];
       record_constants(*r.P, r.p, R, Rb, S.rc);
       S.nx = r.c->nx; S.ny = r.c->ny; S.off = r.c->band_off; S.stamp = r.stamp;
+      if (HELD) S.held = r.c->any_held;
       S.table = band_table(*r.P, S.off, r.p);
       S.i2R = 0.5f / S.rc.r;
       rows = R == Rb ? 2 * S.off + 1 : 0;  // an ellipse has a kernel of its own
@@ -524,7 +532,7 @@ __device__ __forceinline__ void step_group(int n, const Ref& ref, StepShared& sh
       append_to_tiles(*r.TL, r.c->ntx, sh.slot[s].rg, r.p, lane, r.err);
     }
   } else {
-    band_group(sh, n, threadIdx.x - 64);
+    band_group<HELD>(sh, n, threadIdx.x - 64);
   }
 }
 

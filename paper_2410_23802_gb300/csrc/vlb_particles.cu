@@ -12,14 +12,15 @@ __global__ void particle_range_kernel(const ParticleConst c, const ParticleArray
 }
 
 // Lists of every particle and band tables of the disks at the initial state,
-// one warp per particle.
+// one warp per particle.  HELD: of a lattice with held particles.
+template <bool HELD>
 __global__ void __launch_bounds__(32 * BAND_WARPS) particle_band_kernel(const ParticleConst c, const ParticleArrays P,
                                                                         const TileLists TL, unsigned* err) {
   __shared__ int s_queue[BAND_WARPS][BAND_QUEUE];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int p = blockIdx.x * BAND_WARPS + warp;
   if (p >= c.np) return;  // the whole warp
-  band_one(c, P, TL, err, p, c.band_stamp, s_queue[warp], lane);
+  band_one<HELD>(c, P, TL, err, p, c.band_stamp, s_queue[warp], lane);
 }
 
 // Band tables of the ellipses ell[0 .. n - 1], one warp per row.
@@ -36,6 +37,8 @@ __global__ void __launch_bounds__(32 * ELL_WARPS)
 // One particle step (update, then lists and band tables) in one launch: the
 // two depend on the particle alone (see step_group).  `group` particles per
 // CTA.  Ellipses get their band tables from particle_ellipse_kernel after it.
+// HELD: of a lattice with held particles.
+template <bool HELD>
 __global__ void __launch_bounds__(STEP_THREADS) particle_step_kernel(const __grid_constant__ ParticleConst c,
                                                                      const __grid_constant__ ParticleArrays P,
                                                                      const __grid_constant__ TileLists TL,
@@ -43,7 +46,7 @@ __global__ void __launch_bounds__(STEP_THREADS) particle_step_kernel(const __gri
   __shared__ StepShared sh;
   begin_chained();
   const int p0 = blockIdx.x * group;
-  step_group(min(group, c.np - p0), [&](int s) { return StepRef{&c, &P, &TL, err, p0 + s, c.band_stamp}; }, sh);
+  step_group<HELD>(min(group, c.np - p0), [&](int s) { return StepRef{&c, &P, &TL, err, p0 + s, c.band_stamp}; }, sh);
 }
 
 static inline dim3 pgrid(int n) { return dim3((unsigned)((n + 127) / 128)); }
@@ -67,7 +70,7 @@ cudaError_t launch_particle_band(const ParticleConst& c, const ParticleArrays& P
                                  int nell, unsigned* err, cudaStream_t st) {
   if (c.np == 0) return cudaSuccess;
   const unsigned grid = (unsigned)((c.np + BAND_WARPS - 1) / BAND_WARPS);
-  particle_band_kernel<<<grid, 32 * BAND_WARPS, 0, st>>>(c, P, TL, err);
+  (c.any_held ? particle_band_kernel<true> : particle_band_kernel<false>)<<<grid, 32 * BAND_WARPS, 0, st>>>(c, P, TL, err);
   if (const cudaError_t e = cudaGetLastError(); e != cudaSuccess) return e;
   return launch_ellipses(c, P, ell, nell, st);
 }
@@ -75,8 +78,8 @@ cudaError_t launch_particle_step(const ParticleConst& c, const ParticleArrays& P
                                  int nell, unsigned* err, cudaStream_t st) {
   if (c.np == 0) return cudaSuccess;
   const int group = step_group_size(c.np);
-  const cudaError_t e = launch_chained(particle_step_kernel, dim3((unsigned)((c.np + group - 1) / group)),
-                                       dim3(STEP_THREADS), st, c, P, TL, err, group);
+  const cudaError_t e = launch_chained(c.any_held ? particle_step_kernel<true> : particle_step_kernel<false>,
+                                       dim3((unsigned)((c.np + group - 1) / group)), dim3(STEP_THREADS), st, c, P, TL, err, group);
   if (e != cudaSuccess) return e;
   return launch_ellipses(c, P, ell, nell, st);
 }
