@@ -1496,7 +1496,10 @@ uint64_t state_bytes(const StateHeader& H) {
 
 // Population buffer b to (out) or from (in) an image's eighteen planes, a
 // direction at a time: split or joined on the device in two planes of scratch,
-// or on the host where the device has no room for them.
+// or on the host where the device has no room for them.  Everything goes
+// through the handle's stream: a pageable copy into the device on the legacy
+// stream may still be under way when its call returns, and the handle's stream
+// would not wait for it.
 template <class W>
 static void split_on_host(W* pairs, W* f, W* g, size_t n, bool join) {
   for (size_t c = 0; c < n; ++c) {
@@ -1529,9 +1532,11 @@ static cudaError_t copy_populations(vlb_handle* h, int b, char* out, const char*
       if (in) {
         for (int q = 0; q < 2; ++q) std::memcpy(two.get() + q * plane, in + (9 * q + i) * plane, plane);
         split(true);
-        e = cudaMemcpy(dev, pairs.get(), 2 * plane, cudaMemcpyHostToDevice);
+        e = cudaMemcpyAsync(dev, pairs.get(), 2 * plane, cudaMemcpyHostToDevice, h->stream);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);  // (the pairs are written again)
       } else {
-        e = cudaMemcpy(pairs.get(), dev, 2 * plane, cudaMemcpyDeviceToHost);
+        e = cudaMemcpyAsync(pairs.get(), dev, 2 * plane, cudaMemcpyDeviceToHost, h->stream);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
         split(false);
         for (int q = 0; q < 2; ++q) std::memcpy(out + (9 * q + i) * plane, two.get() + q * plane, plane);
       }
@@ -1541,15 +1546,15 @@ static cudaError_t copy_populations(vlb_handle* h, int b, char* out, const char*
   for (int i = 0; i < 9 && e == cudaSuccess; ++i) {
     char* pairs = static_cast<char*>(h->pop[b]) + 2 * plane * i;
     for (int q = 0; q < 2 && in && e == cudaSuccess; ++q)
-      e = cudaMemcpy(scratch + q * plane, in + (9 * q + i) * plane, plane, cudaMemcpyHostToDevice);
+      e = cudaMemcpyAsync(scratch + q * plane, in + (9 * q + i) * plane, plane, cudaMemcpyHostToDevice, h->stream);
     if (e == cudaSuccess)
       e = launch_split_plane(pairs, scratch, scratch + plane, h->plane, h->ssize, in != nullptr, h->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
     for (int q = 0; q < 2 && out && e == cudaSuccess; ++q)
-      e = cudaMemcpy(out + (9 * q + i) * plane, scratch + q * plane, plane, cudaMemcpyDeviceToHost);
+      e = cudaMemcpyAsync(out + (9 * q + i) * plane, scratch + q * plane, plane, cudaMemcpyDeviceToHost, h->stream);
   }
+  const cudaError_t es = cudaStreamSynchronize(h->stream);
   cudaFree(scratch);
-  return e;
+  return e != cudaSuccess ? e : es;
 }
 
 extern "C" {
@@ -1613,7 +1618,7 @@ vlb_status vlb_load_state(vlb_handle* h, const void* buf, uint64_t bytes) {
   CK(h, cudaStreamSynchronize(h->stream));
   const char* o = static_cast<const char*>(buf) + sizeof(StateHeader);
   auto put = [&](void* dst, uint64_t n) -> cudaError_t {
-    cudaError_t e = n ? cudaMemcpy(dst, o, n, cudaMemcpyHostToDevice) : cudaSuccess;
+    cudaError_t e = n ? cudaMemcpyAsync(dst, o, n, cudaMemcpyHostToDevice, h->stream) : cudaSuccess;
     o += n;
     return e;
   };
@@ -1629,6 +1634,7 @@ vlb_status vlb_load_state(vlb_handle* h, const void* buf, uint64_t bytes) {
     CK(h, put(h->TL[b].count, I.tl_count_bytes));
     CK(h, put(h->TL[b].ids, I.tl_ids_bytes));
   }
+  CK(h, cudaStreamSynchronize(h->stream));  // the caller's image may go
   // the held-temperature flags and the ellipses' axes came with the particle block
   if (h->np > 0) {
     CK(h, cudaMemcpy(h->hfix.data(), h->P.fixed_T, h->np * sizeof(int), cudaMemcpyDeviceToHost));

@@ -1,0 +1,24 @@
+"""State images of lattices whose planes are several MB, for every storage type
+(the 2-, 4- and 8-byte forms of the split into planes), at an odd side: a run
+saved and restored into a fresh handle continues bit for bit."""
+import pytest
+
+from helpers import gpu_lattice
+from paper_2410_23802_gb300 import workloads as W
+from test_gpu_checkpoint import _assert_same, _snapshot
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("precision", ["fp16", "bf16", "fp32", "fp64"])
+def test_large_image_resumes_bit_for_bit(precision):
+    case = W.cavity(side=1261, n=40, seed=17)
+    with gpu_lattice(case, precision=precision) as a:
+        a.step(9)
+        img = a.save_state()
+        a.step(8)
+        ref = _snapshot(a)
+    with gpu_lattice(case, precision=precision) as b:
+        b.load_state(img)
+        b.step(8)
+        _assert_same(_snapshot(b), ref)
