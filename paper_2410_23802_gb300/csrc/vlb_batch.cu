@@ -113,28 +113,28 @@ __global__ void __launch_bounds__(32 * ELL_WARPS)
 }
 
 template <class S, class C>
-static cudaError_t launch_batch(const BatchLattice<C>* cases, const int* tile_case, int ntiles, int k, bool held,
-                                cudaStream_t st) {
+static cudaError_t launch_batch(const BatchLattice<C>* cases, const int* tile_case, int ntiles, int k, bool particles,
+                                bool held, cudaStream_t st) {
   constexpr bool HOLD = !std::is_same<S, AnyStorage>::value;  // (held lattices of one launch share their storage)
   if (ntiles == 0) return cudaSuccess;
   constexpr int WARPS = tile_warps<C>();
   const dim3 block(32, WARPS);
   const int per_cta = duty_span(ntiles) * WARPS, duty = (ntiles + per_cta - 1) / per_cta;
   const unsigned grid = (unsigned)duty + (unsigned)ntiles * (TILE_Y / WARPS);
-  return launch_chained(held ? lattice_batch_kernel<S, C, HOLD> : lattice_batch_kernel<S, C, false>, dim3(grid), block,
-                        st, cases, tile_case, ntiles, k, duty);
+  return launch_chained(held ? lattice_batch_kernel<S, C, HOLD> : lattice_batch_kernel<S, C, false>, particles,
+                        dim3(grid), block, st, cases, tile_case, ntiles, k, duty);
 }
 
 cudaError_t launch_lattice_batch_f32(const BatchLattice<float>* cases, const int* tile_case, int ntiles, int k,
-                                     int storage, bool held, cudaStream_t st) {
-  if (storage == STORE_ANY) return launch_batch<AnyStorage, float>(cases, tile_case, ntiles, k, held, st);
-  if (storage == STORE_F16) return launch_batch<__half, float>(cases, tile_case, ntiles, k, held, st);
-  if (storage == STORE_BF16) return launch_batch<__nv_bfloat16, float>(cases, tile_case, ntiles, k, held, st);
-  return launch_batch<float, float>(cases, tile_case, ntiles, k, held, st);
+                                     int storage, bool particles, bool held, cudaStream_t st) {
+  if (storage == STORE_ANY) return launch_batch<AnyStorage, float>(cases, tile_case, ntiles, k, particles, held, st);
+  if (storage == STORE_F16) return launch_batch<__half, float>(cases, tile_case, ntiles, k, particles, held, st);
+  if (storage == STORE_BF16) return launch_batch<__nv_bfloat16, float>(cases, tile_case, ntiles, k, particles, held, st);
+  return launch_batch<float, float>(cases, tile_case, ntiles, k, particles, held, st);
 }
 cudaError_t launch_lattice_batch_f64(const BatchLattice<double>* cases, const int* tile_case, int ntiles, int k,
-                                     bool held, cudaStream_t st) {
-  return launch_batch<double, double>(cases, tile_case, ntiles, k, held, st);
+                                     bool particles, bool held, cudaStream_t st) {
+  return launch_batch<double, double>(cases, tile_case, ntiles, k, particles, held, st);
 }
 
 cudaError_t launch_ellipse_batch(const BatchParticles* cases, const BatchEllipses& ell, int k, const int* kdev,
@@ -142,7 +142,7 @@ cudaError_t launch_ellipse_batch(const BatchParticles* cases, const BatchEllipse
   if (ell.n == 0) return cudaSuccess;
   const int blocks = (ell.rows + ELL_WARPS - 1) / ELL_WARPS;
   const dim3 grid((unsigned)(blocks * ell.n)), block(32 * ELL_WARPS);
-  if (!kdev) return launch_chained(particle_ellipse_batch_kernel, grid, block, st, cases, ell.items, blocks, k, kdev);
+  if (!kdev) return launch_chained(particle_ellipse_batch_kernel, true, grid, block, st, cases, ell.items, blocks, k, kdev);
   // (behind a persistent launch, captured into a graph: an ordinary launch)
   particle_ellipse_batch_kernel<<<grid, block, 0, st>>>(cases, ell.items, blocks, k, kdev);
   return cudaGetLastError();
@@ -151,7 +151,7 @@ cudaError_t launch_particle_step_batch(const BatchParticles* cases, const int2* 
                                        const BatchEllipses& ell, cudaStream_t st) {
   if (nitems == 0) return cudaSuccess;
   const int group = step_group_size(nitems);
-  const cudaError_t e = launch_chained(held ? particle_step_batch_kernel<true> : particle_step_batch_kernel<false>,
+  const cudaError_t e = launch_chained(held ? particle_step_batch_kernel<true> : particle_step_batch_kernel<false>, true,
                                        dim3((unsigned)((nitems + group - 1) / group)), dim3(STEP_THREADS), st, cases, items, nitems, k, group);
   return e != cudaSuccess ? e : launch_ellipse_batch(cases, ell, k, nullptr, st);
 }

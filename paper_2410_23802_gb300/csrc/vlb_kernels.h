@@ -6,18 +6,23 @@
 namespace vlb {
 
 // Launch of a kernel that begins with begin_chained(): behind another kernel
-// of the stream its CTAs are brought in before that one has drained.
+// of the stream its CTAs are brought in before that one has drained.  `early`
+// false: only after it (an ordinary launch).  The lattice kernels take that
+// where no particle kernel lies between them: they read the populations as data
+// that nobody writes while they exist, and the lattice kernel before them still
+// writes those.  (Behind a particle kernel they come in only once that one has
+// passed its own wait, i.e. after the lattice kernel before it.)
 template <class... P, class... A>
-cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t st, A... args) {
-  cudaLaunchAttribute early{};
-  early.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  early.val.programmaticStreamSerializationAllowed = 1;
+cudaError_t launch_chained(void (*kernel)(P...), bool early, dim3 grid, dim3 block, cudaStream_t st, A... args) {
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = grid;
   cfg.blockDim = block;
   cfg.stream = st;
-  cfg.attrs = &early;
-  cfg.numAttrs = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = early ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
 }
 
@@ -94,12 +99,13 @@ cudaError_t launch_particle_step_batch(const BatchParticles* cases, const int2* 
                                        const BatchEllipses& ell, cudaStream_t st);
 
 // Batched step k: lattice tiles map to their case through tile_case.
+// `particles`: a particle kernel precedes (some case of the batch has particles);
 // `held`: the held-temperature path (every case of the launch shares
 // arithmetic, held, and the storage unless that is STORE_ANY, never with held).
 cudaError_t launch_lattice_batch_f32(const BatchLattice<float>* cases, const int* tile_case, int ntiles, int k,
-                                     int storage, bool held, cudaStream_t st);
+                                     int storage, bool particles, bool held, cudaStream_t st);
 cudaError_t launch_lattice_batch_f64(const BatchLattice<double>* cases, const int* tile_case, int ntiles, int k,
-                                     bool held, cudaStream_t st);
+                                     bool particles, bool held, cudaStream_t st);
 
 // The persistent form of a batched step: one launch of a grid the size of the
 // GPU's resident capacity per level.  Its CTAs take work chunks in order from

@@ -61,7 +61,7 @@ static cudaError_t launch_ellipses(const ParticleConst& c, const ParticleArrays&
                                    cudaStream_t st) {
   if (nell > 0) {
     const int blocks = (2 * c.band_off + ELL_WARPS) / ELL_WARPS;  // rows 0 .. 2 band_off
-    return launch_chained(particle_ellipse_kernel, dim3((unsigned)(blocks * nell)), dim3(32 * ELL_WARPS), st, c, P, ell,
+    return launch_chained(particle_ellipse_kernel, true, dim3((unsigned)(blocks * nell)), dim3(32 * ELL_WARPS), st, c, P, ell,
                           blocks);
   }
   return cudaSuccess;
@@ -78,7 +78,7 @@ cudaError_t launch_particle_step(const ParticleConst& c, const ParticleArrays& P
                                  int nell, unsigned* err, cudaStream_t st) {
   if (c.np == 0) return cudaSuccess;
   const int group = step_group_size(c.np);
-  const cudaError_t e = launch_chained(c.any_held ? particle_step_kernel<true> : particle_step_kernel<false>,
+  const cudaError_t e = launch_chained(c.any_held ? particle_step_kernel<true> : particle_step_kernel<false>, true,
                                        dim3((unsigned)((c.np + group - 1) / group)), dim3(STEP_THREADS), st, c, P, TL, err, group);
   if (e != cudaSuccess) return e;
   return launch_ellipses(c, P, ell, nell, st);

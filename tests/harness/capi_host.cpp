@@ -1,0 +1,71 @@
+// Host harness of the C ABI's host code (vlb_capi.cu) over the stand-in for the
+// CUDA runtime of fake_cuda.cpp, where kernels do nothing but split and join
+// population planes.
+//
+// Usage: capi_host CHECK, one of
+//   roundtrip   loads an image of random bytes into handles of each storage type
+//               and saves it again: the two must be equal
+// Prints "ok", or what differs and exits with 1.
+#include <cstdio>
+#include <cstdlib>
+#include <cstring>
+#include <map>
+#include <string>
+#include <vector>
+
+#include "../../include/vlb.h"
+#include "fake_cuda.h"
+
+static int bad(const char* what, int precision) {
+  std::printf("%s (precision %d)\n", what, precision);
+  return 1;
+}
+// A handle of three particles, two of them ellipses, at its initial state.
+static vlb_handle* make(int precision) {
+  vlb_params p;
+  vlb_params_default(&p);
+  p.nx = 61;
+  p.ny = 43;
+  p.precision = precision;
+  p.max_particles = 5;
+  vlb_handle* h = nullptr;
+  const double disk[2] = {12.5, 30.25}, two[4] = {20.0, 12.0, 45.0, 25.0}, a[2] = {6.0, 7.0}, b[2] = {3.0, 4.0};
+  const double theta[2] = {0.3, -0.4}, T0[2] = {0.0, 0.0}, r = 5.0;
+  if (vlb_create(&p, &h) != VLB_OK || vlb_add_particles(h, 1, disk, &r, T0, nullptr, nullptr, nullptr) != VLB_OK ||
+      vlb_add_ellipses(h, 2, two, a, b, theta, T0, nullptr, nullptr, nullptr) != VLB_OK || vlb_step(h, 0) != VLB_OK) {
+    std::printf("setup: %s\n", vlb_last_error(h));
+    std::exit(1);
+  }
+  return h;
+}
+// An image of the handle's shape with random bytes in place of its state.
+static std::vector<char> random_image(vlb_handle* h) {
+  uint64_t n = 0;
+  if (vlb_state_size(h, &n) != VLB_OK) std::exit(bad("state size", -1));
+  std::vector<char> image(n);
+  if (vlb_save_state(h, image.data(), n) != VLB_OK) std::exit(bad("save", -1));
+  uint32_t header = 0, s = 12345;
+  std::memcpy(&header, image.data() + 12, sizeof(header));  // (magic, version, the header's bytes)
+  for (size_t i = header; i < n; ++i) image[i] = (char)((s = s * 1664525u + 1013904223u) >> 24);
+  return image;
+}
+static int roundtrip() {
+  for (int precision : {VLB_FP64, VLB_FP32, VLB_FP16_STORE, VLB_BF16_STORE}) {
+    vlb_handle* h = make(precision);
+    const std::vector<char> image = random_image(h);
+    std::vector<char> again(image.size());
+    if (vlb_load_state(h, image.data(), image.size()) != VLB_OK) return bad(vlb_last_error(h), precision);
+    if (vlb_save_state(h, again.data(), again.size()) != VLB_OK) return bad(vlb_last_error(h), precision);
+    if (again != image) return bad("the saved image differs from the loaded one", precision);
+    vlb_destroy(h);
+  }
+  return 0;
+}
+
+int main(int argc, char** argv) {
+  const std::map<std::string, int (*)()> checks = {{"roundtrip", roundtrip}};
+  const auto it = argc > 1 ? checks.find(argv[1]) : checks.end();
+  if (it == checks.end() || it->second() != 0) return 1;
+  std::printf("ok\n");
+  return 0;
+}

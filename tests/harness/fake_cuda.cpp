@@ -11,6 +11,7 @@
 #include <functional>
 #include <map>
 #include <set>
+#include <string>
 #include <vector>
 
 #include <cuda_runtime_api.h>
@@ -19,9 +20,14 @@ namespace fake {
 size_t live = 0;
 long allocs = 0;
 bool full = false;
+std::vector<Launch> launches;
 }  // namespace fake
 using namespace fake;
 
+static std::map<const void*, std::string>& kernels() {  // names by their host entry (registered before main)
+  static std::map<const void*, std::string> names;
+  return names;
+}
 static std::map<char*, size_t> g_device;        // live device buffers
 static std::set<void*> g_pinned;                // page-locked host buffers
 static std::vector<std::function<void()>> g_legacy;  // writes of the legacy stream still to come
@@ -49,6 +55,18 @@ static cudaError_t device_free(void* p) {
 }
 static void copy2d(void* d, size_t dp, const void* s, size_t sp, size_t w, size_t h) {
   for (size_t y = 0; y < h; ++y) std::memcpy((char*)d + y * dp, (const char*)s + y * sp, w);
+}
+// split_plane_kernel(pairs, f, g, n, join) on words of w bytes
+static void split_plane(void** args, size_t w) {
+  char *q = *(char**)args[0], *f = *(char**)args[1], *g = *(char**)args[2];
+  const long long n = *(long long*)args[3];
+  const bool join = *(int*)args[4] != 0;
+  for (long long c = 0; c < n; ++c) {
+    for (int k = 0; k < 2; ++k) {
+      char *pair = q + (2 * c + k) * w, *one = (k ? g : f) + c * w;
+      std::memcpy(join ? pair : one, join ? one : pair, w);
+    }
+  }
 }
 
 extern "C" {
@@ -107,6 +125,33 @@ cudaError_t cudaGraphExecUpdate(cudaGraphExec_t, cudaGraph_t, cudaGraphExecUpdat
 cudaError_t cudaGraphLaunch(cudaGraphExec_t, cudaStream_t) { return cudaErrorNotSupported; }
 cudaError_t cudaGraphDestroy(cudaGraph_t) { return cudaSuccess; }
 cudaError_t cudaGraphExecDestroy(cudaGraphExec_t) { return cudaSuccess; }
+// kernel launches: recorded, and run if they split or join planes
+cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* cfg, const void* kernel, void**) {
+  bool early = false;
+  for (unsigned k = 0; k < cfg->numAttrs; ++k) early |= cfg->attrs[k].id == cudaLaunchAttributeProgrammaticStreamSerialization;
+  launches.push_back({kernels()[kernel], early});
+  return cudaSuccess;
+}
+cudaError_t __cudaLaunchKernel(cudaKernel_t kernel, dim3, dim3, void** args, size_t, cudaStream_t st) {
+  const std::string& name = kernels()[(const void*)kernel];
+  launches.push_back({name, false});
+  if (!st) legacy_wait();
+  if (name.find("split_plane_kernelIyE") != name.npos) split_plane(args, 8);
+  if (name.find("split_plane_kernelIjE") != name.npos) split_plane(args, 4);
+  if (name.find("split_plane_kernelItE") != name.npos) split_plane(args, 2);
+  return cudaSuccess;
+}
+cudaError_t __cudaGetKernel(cudaKernel_t* k, const void* f) { *k = (cudaKernel_t)f; return cudaSuccess; }
+unsigned __cudaPushCallConfiguration(dim3, dim3, size_t, void*) { return 0; }
+cudaError_t __cudaPopCallConfiguration(dim3*, dim3*, size_t*, void*) { return cudaSuccess; }
+void __cudaRegisterFunction(void**, const char* host, char*, const char* name, int, uint3*, uint3*, dim3*, dim3*, int*) {
+  kernels()[host] = name;
+}
+cudaError_t cudaDeviceGetAttribute(int* v, cudaDeviceAttr, int) { *v = 1; return cudaSuccess; }
+cudaError_t cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int* n, const void*, int, size_t, unsigned) {
+  *n = 1;
+  return cudaSuccess;
+}
 void** __cudaRegisterFatBinary(void*) { static void* h; return &h; }
 void __cudaRegisterFatBinaryEnd(void**) {}
 void __cudaUnregisterFatBinary(void**) {}
