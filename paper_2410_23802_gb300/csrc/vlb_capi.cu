@@ -61,8 +61,7 @@ struct vlb_handle {
   int tl = 0;  // list buffer of the current level
   void* pbase = nullptr;
   size_t pbytes = 0;  // bytes of the particle block at pbase
-  int* ell = nullptr;  // the particles that are ellipses, on the device (null: none)
-  int nell = 0;
+  int nell = 0;       // particles that are ellipses
   // device error word and its pinned host copy (refreshed in stream order)
   unsigned* err_host = nullptr;
   bool err_host_external = false;  // the served mode's arena owns it
@@ -225,7 +224,6 @@ static void free_all(vlb_handle* h) {
     dev_free(h, h->TL[b].count);
     dev_free(h, h->TL[b].ids);
   }
-  dev_free(h, h->ell);
   dev_free(h, h->P.mes);
   dev_free(h, h->P.band);
   dev_free(h, h->audit_scratch);
@@ -611,16 +609,16 @@ static vlb_status upload_particles(vlb_handle* h, int first, int count) {
   return VLB_OK;
 }
 
-// The list of the ellipses (after the host's axes are known).
+// The list of the ellipses (after the host's axes are known), into the rows of
+// P.pk: the bytes that a handle allocates are the same with and without it.
 static vlb_status upload_ellipses(vlb_handle* h) {
-  std::vector<int> ids;
+  std::vector<double> ids;
   for (int k = 0; k < h->np; ++k)
     if (h->hrb[k] != h->hr[k]) ids.push_back(k);
   h->nell = (int)ids.size();
   if (ids.empty()) return VLB_OK;
-  // (room for every particle: a loaded state may hold other axes)
-  if (!h->ell) CK(h, dev_alloc(h, reinterpret_cast<void**>(&h->ell), (size_t)std::max(h->cap, 1) * sizeof(int)));
-  CK(h, cudaMemcpyAsync(h->ell, ids.data(), ids.size() * sizeof(int), cudaMemcpyHostToDevice, h->stream));
+  CK(h, cudaMemcpy2DAsync(h->P.pk + 6, 8 * sizeof(double), ids.data(), sizeof(double), sizeof(double), ids.size(),
+                          cudaMemcpyHostToDevice, h->stream));
   CK(h, cudaStreamSynchronize(h->stream));  // the list on the host ends here
   return VLB_OK;
 }
@@ -672,7 +670,7 @@ static vlb_status initialize(vlb_handle* h) {
   h->tl = 0;
   next_band_stamp(h);
   if (vlb_status st = upload_ellipses(h); st != VLB_OK) return st;
-  CK(h, launch_particle_band(c, h->P, h->TL[0], h->ell, h->nell, h->err_dev, h->stream));
+  CK(h, launch_particle_band(c, h->P, h->TL[0], h->nell, h->err_dev, h->stream));
   h->cur = 0;
   vlb_status s = launch_lattice(h, MODE_INIT, 0, 0, 0);
   if (s != VLB_OK) return s;
@@ -687,7 +685,7 @@ static vlb_status step_once(vlb_handle* h) {
   vlb_status s;
   const int nl = 1 - h->tl;
   next_band_stamp(h);
-  CK(h, launch_particle_step(h->PC, h->P, h->TL[nl], h->ell, h->nell, h->err_dev, h->stream));
+  CK(h, launch_particle_step(h->PC, h->P, h->TL[nl], h->nell, h->err_dev, h->stream));
   const bool rec = h->prof && h->ev_used + 2 <= h->ev_cap;
   if (rec) CK(h, cudaEventRecord(h->ev[h->ev_used], h->stream));
   if ((s = launch_lattice(h, MODE_STEP, h->cur, 1 - h->cur, nl)) != VLB_OK) return s;

@@ -93,7 +93,8 @@ struct ParticleArrays {
   int* nbr_count;          // contact partners per particle
   int* nbr;                // [n][NBR_CAP], unordered (sorted where used)
   int* fixed_T;            // [n] held at T0: 1 over the covered part (reading R11), 2 whole cells (R11b)
-  double* pk;              // [n][8] constants: 1/M, 1/I, M_in, I_in, body force factor, wall factor
+  double* pk;              // [n][8] constants: 1/M, 1/I, M_in, I_in, body force factor, wall factor; and in
+                           // [i][6] the id of the i-th ellipse
   RasterRec* rec;          // [n] raster records of the current level
   int2* band;              // [n][bw][bw] band tables: (class | stamp << 2, area bits) of the cells of
                            // each disk's box, bw = 2 band_off + 1, centred on the record's cell

@@ -79,16 +79,16 @@ cudaError_t launch_raster_dump_f64(const LatticeConst<double>& K, const Particle
                                    const TileLists& TL, unsigned char* count, int* owner,
                                    unsigned char* flag, double* fsp, unsigned* err, cudaStream_t st);
 
-// Particle step pieces (ell[nell]: the particles that are ellipses, on the device).
+// Particle step pieces (nell: the particles that are ellipses).
 cudaError_t launch_particle_range(const ParticleConst& c, const ParticleArrays& P, unsigned* err,
                                   cudaStream_t st);
-cudaError_t launch_particle_band(const ParticleConst& c, const ParticleArrays& P, const TileLists& TL, const int* ell,
-                                 int nell, unsigned* err, cudaStream_t st);
+cudaError_t launch_particle_band(const ParticleConst& c, const ParticleArrays& P, const TileLists& TL, int nell,
+                                 unsigned* err, cudaStream_t st);
 
 // Update, lists and band tables of every particle (list buffer TL, the stamp
 // of ParticleConst).
-cudaError_t launch_particle_step(const ParticleConst& c, const ParticleArrays& P, const TileLists& TL, const int* ell,
-                                 int nell, unsigned* err, cudaStream_t st);
+cudaError_t launch_particle_step(const ParticleConst& c, const ParticleArrays& P, const TileLists& TL, int nell,
+                                 unsigned* err, cudaStream_t st);
 // The (case, ellipse) pairs of a batch, on the device, and the most rows of their boxes.
 struct BatchEllipses {
   const int2* items;

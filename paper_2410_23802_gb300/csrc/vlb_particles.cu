@@ -23,15 +23,15 @@ __global__ void __launch_bounds__(32 * BAND_WARPS) particle_band_kernel(const Pa
   band_one<HELD>(c, P, TL, err, p, c.band_stamp, s_queue[warp], lane);
 }
 
-// Band tables of the ellipses ell[0 .. n - 1], one warp per row.
+// Band tables of the ellipses (their ids: see ParticleArrays::pk), one warp per row.
 __global__ void __launch_bounds__(32 * ELL_WARPS)
-    particle_ellipse_kernel(const ParticleConst c, const ParticleArrays P, const int* __restrict__ ell, int blocks) {
+    particle_ellipse_kernel(const ParticleConst c, const ParticleArrays P, int blocks) {
   __shared__ int s_queue[ELL_WARPS][32];
   begin_chained();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int i = blockIdx.x / blocks, by = (blockIdx.x - i * blocks) * ELL_WARPS + warp;
   if (by >= 2 * c.band_off + 1) return;  // the whole warp
-  ellipse_row(c, P, ell[i], c.band_stamp, by, lane, s_queue[warp]);
+  ellipse_row(c, P, (int)P.pk[8 * (long long)i + 6], c.band_stamp, by, lane, s_queue[warp]);
 }
 
 // One particle step (update, then lists and band tables) in one launch: the
@@ -57,30 +57,29 @@ cudaError_t launch_particle_range(const ParticleConst& c, const ParticleArrays& 
   particle_range_kernel<<<pgrid(c.np), 128, 0, st>>>(c, P, err);
   return cudaGetLastError();
 }
-static cudaError_t launch_ellipses(const ParticleConst& c, const ParticleArrays& P, const int* ell, int nell,
-                                   cudaStream_t st) {
+static cudaError_t launch_ellipses(const ParticleConst& c, const ParticleArrays& P, int nell, cudaStream_t st) {
   if (nell > 0) {
     const int blocks = (2 * c.band_off + ELL_WARPS) / ELL_WARPS;  // rows 0 .. 2 band_off
-    return launch_chained(particle_ellipse_kernel, true, dim3((unsigned)(blocks * nell)), dim3(32 * ELL_WARPS), st, c, P, ell,
+    return launch_chained(particle_ellipse_kernel, true, dim3((unsigned)(blocks * nell)), dim3(32 * ELL_WARPS), st, c, P,
                           blocks);
   }
   return cudaSuccess;
 }
-cudaError_t launch_particle_band(const ParticleConst& c, const ParticleArrays& P, const TileLists& TL, const int* ell,
-                                 int nell, unsigned* err, cudaStream_t st) {
+cudaError_t launch_particle_band(const ParticleConst& c, const ParticleArrays& P, const TileLists& TL, int nell,
+                                 unsigned* err, cudaStream_t st) {
   if (c.np == 0) return cudaSuccess;
   const unsigned grid = (unsigned)((c.np + BAND_WARPS - 1) / BAND_WARPS);
   (c.any_held ? particle_band_kernel<true> : particle_band_kernel<false>)<<<grid, 32 * BAND_WARPS, 0, st>>>(c, P, TL, err);
   if (const cudaError_t e = cudaGetLastError(); e != cudaSuccess) return e;
-  return launch_ellipses(c, P, ell, nell, st);
+  return launch_ellipses(c, P, nell, st);
 }
-cudaError_t launch_particle_step(const ParticleConst& c, const ParticleArrays& P, const TileLists& TL, const int* ell,
-                                 int nell, unsigned* err, cudaStream_t st) {
+cudaError_t launch_particle_step(const ParticleConst& c, const ParticleArrays& P, const TileLists& TL, int nell,
+                                 unsigned* err, cudaStream_t st) {
   if (c.np == 0) return cudaSuccess;
   const int group = step_group_size(c.np);
   const cudaError_t e = launch_chained(c.any_held ? particle_step_kernel<true> : particle_step_kernel<false>, true,
                                        dim3((unsigned)((c.np + group - 1) / group)), dim3(STEP_THREADS), st, c, P, TL, err, group);
   if (e != cudaSuccess) return e;
-  return launch_ellipses(c, P, ell, nell, st);
+  return launch_ellipses(c, P, nell, st);
 }
 }  // namespace vlb

@@ -5,6 +5,8 @@
 // Usage: capi_host CHECK, one of
 //   roundtrip   loads an image of random bytes into handles of each storage type
 //               and saves it again: the two must be equal
+//   footprint   device bytes of a handle with ellipses and one without, after
+//               the first step: what vlb_device_bytes says
 // Prints "ok", or what differs and exits with 1.
 #include <cstdio>
 #include <cstdlib>
@@ -20,8 +22,9 @@ static int bad(const char* what, int precision) {
   std::printf("%s (precision %d)\n", what, precision);
   return 1;
 }
-// A handle of three particles, two of them ellipses, at its initial state.
-static vlb_handle* make(int precision) {
+// A handle of three particles, two of them ellipses unless `disks`, at its
+// initial state.
+static vlb_handle* make(int precision, bool disks = false, uint64_t* bytes = nullptr) {
   vlb_params p;
   vlb_params_default(&p);
   p.nx = 61;
@@ -30,9 +33,10 @@ static vlb_handle* make(int precision) {
   p.max_particles = 5;
   vlb_handle* h = nullptr;
   const double disk[2] = {12.5, 30.25}, two[4] = {20.0, 12.0, 45.0, 25.0}, a[2] = {6.0, 7.0}, b[2] = {3.0, 4.0};
-  const double theta[2] = {0.3, -0.4}, T0[2] = {0.0, 0.0}, r = 5.0;
+  const double theta[2] = {0.3, -0.4}, T0[2] = {0.0, 0.0}, r = 5.0, radius[3] = {5.0, 6.0, 7.0};
+  if (bytes) vlb_device_bytes(&p, 3, radius, bytes);
   if (vlb_create(&p, &h) != VLB_OK || vlb_add_particles(h, 1, disk, &r, T0, nullptr, nullptr, nullptr) != VLB_OK ||
-      vlb_add_ellipses(h, 2, two, a, b, theta, T0, nullptr, nullptr, nullptr) != VLB_OK || vlb_step(h, 0) != VLB_OK) {
+      vlb_add_ellipses(h, 2, two, a, disks ? a : b, theta, T0, nullptr, nullptr, nullptr) != VLB_OK || vlb_step(h, 0) != VLB_OK) {
     std::printf("setup: %s\n", vlb_last_error(h));
     std::exit(1);
   }
@@ -46,7 +50,11 @@ static std::vector<char> random_image(vlb_handle* h) {
   if (vlb_save_state(h, image.data(), n) != VLB_OK) std::exit(bad("save", -1));
   uint32_t header = 0, s = 12345;
   std::memcpy(&header, image.data() + 12, sizeof(header));  // (magic, version, the header's bytes)
-  for (size_t i = header; i < n; ++i) image[i] = (char)((s = s * 1664525u + 1013904223u) >> 24);
+  // (the populations and S; what follows says which particles are ellipses)
+  uint64_t sizes[2];
+  std::memcpy(sizes, image.data() + 72, sizeof(sizes));
+  const size_t end = header + 2 * (sizes[0] + sizes[1]);
+  for (size_t i = header; i < end; ++i) image[i] = (char)((s = s * 1664525u + 1013904223u) >> 24);
   return image;
 }
 static int roundtrip() {
@@ -62,8 +70,23 @@ static int roundtrip() {
   return 0;
 }
 
+static int footprint() {
+  for (int precision : {VLB_FP64, VLB_FP32, VLB_FP16_STORE, VLB_BF16_STORE}) {
+    for (bool disks : {true, false}) {
+      uint64_t bytes = 0;
+      const size_t before = fake::live;
+      vlb_handle* h = make(precision, disks, &bytes);
+      if (vlb_step(h, 2) != VLB_OK) return bad(vlb_last_error(h), precision);
+      if (fake::live - before != bytes) return bad(disks ? "disks: other bytes" : "ellipses: other bytes", precision);
+      vlb_destroy(h);
+      if (fake::live != before) return bad("bytes left behind", precision);
+    }
+  }
+  return 0;
+}
+
 int main(int argc, char** argv) {
-  const std::map<std::string, int (*)()> checks = {{"roundtrip", roundtrip}};
+  const std::map<std::string, int (*)()> checks = {{"roundtrip", roundtrip}, {"footprint", footprint}};
   const auto it = argc > 1 ? checks.find(argv[1]) : checks.end();
   if (it == checks.end() || it->second() != 0) return 1;
   std::printf("ok\n");

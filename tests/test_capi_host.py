@@ -20,3 +20,7 @@ def _check(harness, name):
 
 def test_loaded_image_is_saved_again(harness):
     _check(harness, "roundtrip")
+
+
+def test_device_bytes_counts_every_allocation(harness):
+    _check(harness, "footprint")
