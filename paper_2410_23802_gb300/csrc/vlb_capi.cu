@@ -1493,54 +1493,26 @@ uint64_t state_bytes(const StateHeader& H) {
 }  // extern "C"
 
 // Population buffer b to (out) or from (in) an image's eighteen planes, a
-// direction at a time: split or joined on the device in two planes of scratch,
-// or on the host where the device has no room for them.  Everything goes
-// through the handle's stream: a pageable copy into the device on the legacy
-// stream may still be under way when its call returns, and the handle's stream
-// would not wait for it.
-template <class W>
-static void split_on_host(W* pairs, W* f, W* g, size_t n, bool join) {
-  for (size_t c = 0; c < n; ++c) {
-    if (join) {
-      pairs[2 * c] = f[c];
-      pairs[2 * c + 1] = g[c];
-    } else {
-      f[c] = pairs[2 * c];
-      g[c] = pairs[2 * c + 1];
-    }
-  }
-}
+// direction at a time, split or joined on the device.  The two planes of scratch
+// that takes are the macroscopic planes, which the next read-back computes again:
+// an image allocates nothing.  Those of the initial state cannot be computed
+// again; there the other population buffer serves, which no step has written
+// (its part of the image is zero).  Everything goes through the handle's
+// stream: a pageable copy into the device on the legacy stream may still be
+// under way when its call returns, and the handle's stream would not wait for it.
 static cudaError_t copy_populations(vlb_handle* h, int b, char* out, const char* in) {
-  const size_t n = (size_t)h->plane, plane = n * h->ssize;
-  char* scratch = nullptr;
-  cudaError_t e = cudaMalloc(reinterpret_cast<void**>(&scratch), 2 * plane);
-  if (e == cudaErrorMemoryAllocation) {
-    cudaGetLastError();
-    std::unique_ptr<char[]> pairs(new (std::nothrow) char[2 * plane]), two(new (std::nothrow) char[2 * plane]);
-    if (!pairs || !two) return e;
-    auto split = [&](bool join) {
-      char *q = pairs.get(), *f = two.get(), *g = f + plane;
-      if (h->ssize == 8) split_on_host((uint64_t*)q, (uint64_t*)f, (uint64_t*)g, n, join);
-      else if (h->ssize == 4) split_on_host((uint32_t*)q, (uint32_t*)f, (uint32_t*)g, n, join);
-      else split_on_host((uint16_t*)q, (uint16_t*)f, (uint16_t*)g, n, join);
-    };
-    e = cudaSuccess;
-    for (int i = 0; i < 9 && e == cudaSuccess; ++i) {
-      char* dev = static_cast<char*>(h->pop[b]) + 2 * plane * i;
-      if (in) {
-        for (int q = 0; q < 2; ++q) std::memcpy(two.get() + q * plane, in + (9 * q + i) * plane, plane);
-        split(true);
-        e = cudaMemcpyAsync(dev, pairs.get(), 2 * plane, cudaMemcpyHostToDevice, h->stream);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);  // (the pairs are written again)
-      } else {
-        e = cudaMemcpyAsync(pairs.get(), dev, 2 * plane, cudaMemcpyDeviceToHost, h->stream);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
-        split(false);
-        for (int q = 0; q < 2; ++q) std::memcpy(out + (9 * q + i) * plane, two.get() + q * plane, plane);
-      }
+  const size_t plane = (size_t)h->plane * h->ssize;
+  char* scratch = static_cast<char*>(h->macro);
+  if (out && h->step == 0 && h->macros_valid) {
+    if (b != h->cur) {
+      std::memset(out, 0, 18 * plane);
+      return cudaSuccess;
     }
-    return e;
+    scratch = static_cast<char*>(h->pop[1 - b]);
+  } else {
+    h->macros_valid = false;
   }
+  cudaError_t e = cudaSuccess;
   for (int i = 0; i < 9 && e == cudaSuccess; ++i) {
     char* pairs = static_cast<char*>(h->pop[b]) + 2 * plane * i;
     for (int q = 0; q < 2 && in && e == cudaSuccess; ++q)
@@ -1551,7 +1523,6 @@ static cudaError_t copy_populations(vlb_handle* h, int b, char* out, const char*
       e = cudaMemcpyAsync(out + (9 * q + i) * plane, scratch + q * plane, plane, cudaMemcpyDeviceToHost, h->stream);
   }
   const cudaError_t es = cudaStreamSynchronize(h->stream);
-  cudaFree(scratch);
   return e != cudaSuccess ? e : es;
 }
 
@@ -1614,6 +1585,7 @@ vlb_status vlb_load_state(vlb_handle* h, const void* buf, uint64_t bytes) {
   if (bytes < state_bytes(I)) return fail(h, VLB_EINVAL, "vlb_load_state: truncated state image");
   if (I.cur < 0 || I.cur > 1 || I.tl < 0 || I.tl > 1) return fail(h, VLB_EINVAL, "vlb_load_state: corrupt header");
   CK(h, cudaStreamSynchronize(h->stream));
+  h->macros_valid = false;
   const char* o = static_cast<const char*>(buf) + sizeof(StateHeader);
   auto put = [&](void* dst, uint64_t n) -> cudaError_t {
     cudaError_t e = n ? cudaMemcpyAsync(dst, o, n, cudaMemcpyHostToDevice, h->stream) : cudaSuccess;
@@ -1648,7 +1620,6 @@ vlb_status vlb_load_state(vlb_handle* h, const void* buf, uint64_t bytes) {
   h->step = I.step;
   h->PC.band_stamp = I.band_stamp;
   h->K32.band_stamp = h->K64.band_stamp = I.band_stamp;
-  h->macros_valid = false;
   return VLB_OK;
 }
 

@@ -5,6 +5,9 @@
 // Usage: capi_host CHECK, one of
 //   roundtrip   loads an image of random bytes into handles of each storage type
 //               and saves it again: the two must be equal
+//   full        the same with no device memory left, fields read in between, at
+//               step 0 and later: no device allocation, the populations of the
+//               level unchanged
 //   footprint   device bytes of a handle with ellipses and one without, after
 //               the first step: what vlb_device_bytes says
 // Prints "ok", or what differs and exits with 1.
@@ -70,6 +73,39 @@ static int roundtrip() {
   return 0;
 }
 
+static int full() {
+  for (int precision : {VLB_FP64, VLB_FP32, VLB_FP16_STORE, VLB_BF16_STORE}) {
+    vlb_handle* h = make(precision);
+    std::vector<char> image = random_image(h), again(image.size());
+    const long allocs = fake::allocs;
+    if (vlb_load_state(h, image.data(), image.size()) != VLB_OK ||
+        vlb_save_state(h, again.data(), again.size()) != VLB_OK || fake::allocs != allocs)
+      return bad("an image allocated device memory", precision);
+    fake::full = true;
+    std::vector<double> T(61 * 43);
+    for (int step : {0, 7}) {
+      const int64_t at = step;
+      std::memcpy(image.data() + 64, &at, sizeof(at));
+      if (vlb_load_state(h, image.data(), image.size()) != VLB_OK) return bad(vlb_last_error(h), precision);
+      for (int times = 0; times < 3; ++times) {
+        // (a read-back leaves valid macroscopic planes; at step 0 the other
+        // population buffer then has no content)
+        if (vlb_get_fields(h, VLB_FIELD_T, nullptr, nullptr, nullptr, T.data(), nullptr) != VLB_OK)
+          return bad(vlb_last_error(h), precision);
+        if (vlb_save_state(h, again.data(), again.size()) != VLB_OK) return bad(vlb_last_error(h), precision);
+        uint32_t header = 0;
+        uint64_t pop = 0;
+        std::memcpy(&header, image.data() + 12, sizeof(header));
+        std::memcpy(&pop, image.data() + 72, sizeof(pop));
+        if (std::memcmp(again.data() + header, image.data() + header, pop) != 0) return bad("populations changed", precision);
+        if (step > 0 && again != image) return bad("the saved image differs", precision);
+      }
+    }
+    fake::full = false;
+    vlb_destroy(h);
+  }
+  return 0;
+}
 static int footprint() {
   for (int precision : {VLB_FP64, VLB_FP32, VLB_FP16_STORE, VLB_BF16_STORE}) {
     for (bool disks : {true, false}) {
@@ -86,7 +122,7 @@ static int footprint() {
 }
 
 int main(int argc, char** argv) {
-  const std::map<std::string, int (*)()> checks = {{"roundtrip", roundtrip}, {"footprint", footprint}};
+  const std::map<std::string, int (*)()> checks = {{"roundtrip", roundtrip}, {"full", full}, {"footprint", footprint}};
   const auto it = argc > 1 ? checks.find(argv[1]) : checks.end();
   if (it == checks.end() || it->second() != 0) return 1;
   std::printf("ok\n");

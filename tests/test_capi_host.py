@@ -24,3 +24,7 @@ def test_loaded_image_is_saved_again(harness):
 
 def test_device_bytes_counts_every_allocation(harness):
     _check(harness, "footprint")
+
+
+def test_images_allocate_nothing_on_the_device(harness):
+    _check(harness, "full")
