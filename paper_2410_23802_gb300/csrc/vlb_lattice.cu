@@ -95,8 +95,8 @@ __global__ void audit_blocks_kernel(const LatticeConst<C> K, const typename Stor
     double cf = 1.0;
     for (int i = 0; i < 9; ++i) {
       const typename StoredPair<S>::type fg = pop[(long long)i * K.plane + cell];
-      const double v = double(stored_value<float, S>(fg.x));
-      const double w = double(stored_value<float, S>(fg.y));
+      const double v = double(stored_value<C, S>(fg.x));
+      const double w = double(stored_value<C, S>(fg.y));
       bad |= !(v == v) || !(w == w);
       cf += v;
     }

@@ -1,0 +1,34 @@
+"""The audit's total mass against the sum of the populations themselves, taken
+from a state image and added up exactly (fsum).  The audit adds in FP64, in
+sums of at most about 700 terms one after the other (9 populations of a cell,
+the cells of a thread, the threads of a block, 608 blocks), each of which rounds
+within half a unit of the running sum: 700 x 1.2e-16 of the total."""
+import math
+
+import numpy as np
+import pytest
+
+from helpers import gpu_lattice
+from paper_2410_23802_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+def test_mass_is_the_sum_of_the_populations(precision):
+    case = W.cavity(side=157, n=8, seed=3)
+    prm = dict(case.params, gravity=(0.0, -2e-4))  # (a flow of some 1e-2, so that f is far from w)
+    case.params = prm
+    with gpu_lattice(case, precision=precision) as lat:
+        lat.step(60)
+        mass = lat.audit()[0]
+        img = np.frombuffer(bytes(lat.save_state()), dtype=np.uint8)
+    header = int(img[12:16].view(np.uint32)[0])
+    nx, ny, pitch = (int(v) for v in img[16:28].view(np.int32))
+    cur = int(img[48:52].view(np.int32)[0])
+    pop_bytes, s_bytes = (int(v) for v in img[72:88].view(np.uint64))
+    at = header + cur * (pop_bytes + s_bytes)
+    f = img[at:at + pop_bytes].view(np.float64 if precision == "fp64" else np.float32)
+    f = f.reshape(18, ny, pitch)[:9, :, :nx].astype(np.float64)
+    want = math.fsum([float(nx * ny), *f.ravel().tolist()])
+    assert abs(mass - want) <= 700 * 1.2e-16 * want, (mass, want)
