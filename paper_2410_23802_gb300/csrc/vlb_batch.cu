@@ -113,7 +113,7 @@ __global__ void __launch_bounds__(32 * ELL_WARPS)
 }
 
 template <class S, class C>
-static cudaError_t launch_batch(const BatchLattice<C>* cases, const int* tile_case, int ntiles, int k, bool particles,
+static cudaError_t launch_batch(const BatchLattice<C>* cases, const int* tile_case, int ntiles, int k, int particles,
                                 bool held, cudaStream_t st) {
   constexpr bool HOLD = !std::is_same<S, AnyStorage>::value;  // (held lattices of one launch share their storage)
   if (ntiles == 0) return cudaSuccess;
@@ -121,19 +121,19 @@ static cudaError_t launch_batch(const BatchLattice<C>* cases, const int* tile_ca
   const dim3 block(32, WARPS);
   const int per_cta = duty_span(ntiles) * WARPS, duty = (ntiles + per_cta - 1) / per_cta;
   const unsigned grid = (unsigned)duty + (unsigned)ntiles * (TILE_Y / WARPS);
-  return launch_chained(held ? lattice_batch_kernel<S, C, HOLD> : lattice_batch_kernel<S, C, false>, particles,
-                        dim3(grid), block, st, cases, tile_case, ntiles, k, duty);
+  return launch_chained(held ? lattice_batch_kernel<S, C, HOLD> : lattice_batch_kernel<S, C, false>,
+                        lattice_early(particles, ntiles), dim3(grid), block, st, cases, tile_case, ntiles, k, duty);
 }
 
 cudaError_t launch_lattice_batch_f32(const BatchLattice<float>* cases, const int* tile_case, int ntiles, int k,
-                                     int storage, bool particles, bool held, cudaStream_t st) {
+                                     int storage, int particles, bool held, cudaStream_t st) {
   if (storage == STORE_ANY) return launch_batch<AnyStorage, float>(cases, tile_case, ntiles, k, particles, held, st);
   if (storage == STORE_F16) return launch_batch<__half, float>(cases, tile_case, ntiles, k, particles, held, st);
   if (storage == STORE_BF16) return launch_batch<__nv_bfloat16, float>(cases, tile_case, ntiles, k, particles, held, st);
   return launch_batch<float, float>(cases, tile_case, ntiles, k, particles, held, st);
 }
 cudaError_t launch_lattice_batch_f64(const BatchLattice<double>* cases, const int* tile_case, int ntiles, int k,
-                                     bool particles, bool held, cudaStream_t st) {
+                                     int particles, bool held, cudaStream_t st) {
   return launch_batch<double, double>(cases, tile_case, ntiles, k, particles, held, st);
 }
 

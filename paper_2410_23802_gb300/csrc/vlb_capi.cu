@@ -1026,9 +1026,9 @@ static vlb_status step_batch_impl(vlb_handle* const* hs, int32_t n, int32_t nste
         if (e != cudaSuccess) break;
         const int* table = reinterpret_cast<const int*>(dev + g.table_off);
         e = g.f64 ? launch_lattice_batch_f64(reinterpret_cast<const BatchLattice<double>*>(dev + g.desc_off), table,
-                                             g.ntiles, k, nitems > 0, g.held, bs)
+                                             g.ntiles, k, nitems, g.held, bs)
                   : launch_lattice_batch_f32(reinterpret_cast<const BatchLattice<float>*>(dev + g.desc_off), table,
-                                             g.ntiles, k, g.storage, nitems > 0, g.held, bs);
+                                             g.ntiles, k, g.storage, nitems, g.held, bs);
       }
     }
   } else if (e == cudaSuccess) {

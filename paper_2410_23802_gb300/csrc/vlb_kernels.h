@@ -7,11 +7,7 @@ namespace vlb {
 
 // Launch of a kernel that begins with begin_chained(): behind another kernel
 // of the stream its CTAs are brought in before that one has drained.  `early`
-// false: only after it (an ordinary launch).  The lattice kernels take that
-// where no particle kernel lies between them: they read the populations as data
-// that nobody writes while they exist, and the lattice kernel before them still
-// writes those.  (Behind a particle kernel they come in only once that one has
-// passed its own wait, i.e. after the lattice kernel before it.)
+// false: only after it (an ordinary launch).
 template <class... P, class... A>
 cudaError_t launch_chained(void (*kernel)(P...), bool early, dim3 grid, dim3 block, cudaStream_t st, A... args) {
   cudaLaunchAttribute attr{};
@@ -24,6 +20,25 @@ cudaError_t launch_chained(void (*kernel)(P...), bool early, dim3 grid, dim3 blo
   cfg.attrs = &attr;
   cfg.numAttrs = early ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
+// Whether a lattice kernel over `tiles` tiles may come in while the kernel before
+// it runs, with `particles` in the particle kernel of the step.
+//   * Without particles the kernel before is a lattice kernel, which still writes
+//     the populations; they are read as data that nobody writes while the reader
+//     exists.  (A particle kernel lets the lattice kernel in only after its own
+//     wait, i.e. once the lattice kernel before it is done.)
+//   * Crowded lattices: the waiting CTAs take the room that the particle kernel's
+//     CTAs leave.  Where those are more than two per SM and the tiles about as
+//     many, they come to stand many to an SM on some and few on the others, and
+//     the particle tiles' long chains follow one another there.  us per step,
+//     early / ordinary: 4096 disks of R = 2 on 1484 tiles 61.7 / 37.0, 1024 on 378
+//     29.4 / 18.8, 4096 of R = 4 on 3740 55.6 / 39.5, 512 on 504 17.2 / 14.8; on the
+//     other side of the line 2048 of R = 2 on 2888 20.9 / 22.9, 256 on 112 17.3 /
+//     16.8, 256 of R = 4 on 264 13.6 / 14.8, 4096 of R = 8 on 11324 81.8 / 83.7.
+constexpr int CROWD = 304;  // two particle CTAs per SM
+inline bool lattice_early(long long particles, long long tiles) {
+  return particles > 0 && (particles <= CROWD || 4 * tiles >= 5 * particles);
 }
 
 // Constants of the particle kernels (Sec. 2.3 and the contact model).
@@ -99,13 +114,13 @@ cudaError_t launch_particle_step_batch(const BatchParticles* cases, const int2* 
                                        const BatchEllipses& ell, cudaStream_t st);
 
 // Batched step k: lattice tiles map to their case through tile_case.
-// `particles`: a particle kernel precedes (some case of the batch has particles);
+// `particles`: those of every case of the batch (see lattice_early);
 // `held`: the held-temperature path (every case of the launch shares
 // arithmetic, held, and the storage unless that is STORE_ANY, never with held).
 cudaError_t launch_lattice_batch_f32(const BatchLattice<float>* cases, const int* tile_case, int ntiles, int k,
-                                     int storage, bool particles, bool held, cudaStream_t st);
+                                     int storage, int particles, bool held, cudaStream_t st);
 cudaError_t launch_lattice_batch_f64(const BatchLattice<double>* cases, const int* tile_case, int ntiles, int k,
-                                     bool particles, bool held, cudaStream_t st);
+                                     int particles, bool held, cudaStream_t st);
 
 // The persistent form of a batched step: one launch of a grid the size of the
 // GPU's resident capacity per level.  Its CTAs take work chunks in order from

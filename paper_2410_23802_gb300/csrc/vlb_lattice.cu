@@ -134,7 +134,8 @@ static cudaError_t launch_mode(int mode, const LatticeConst<C>& K, const StepBuf
   const int duty_ctas = (ntiles + per_cta - 1) / per_cta;
   const int duty = mode != MODE_MACROS && K.np > 0 ? (duty_ctas + across - 1) / across : 0;
   const dim3 grid(across, K.nty + duty), block(32, WARPS);
-  auto go = [&](auto kernel) { return launch_chained(kernel, K.np > 0, grid, block, st, K, B, P, TL, duty); };
+  const bool early = lattice_early(K.np, ntiles);
+  auto go = [&](auto kernel) { return launch_chained(kernel, early, grid, block, st, K, B, P, TL, duty); };
   // kernels with the held-temperature path only where some particle is held
   // (FP64 holds nothing at the initial state, which is an equilibrium)
   if (mode == MODE_INIT)

@@ -31,3 +31,11 @@ def test_kernels_behind_particle_kernels_come_in_early(launches, run):
     assert all(early for _, early in launches[run + "1"])
     per_step = {"alone": ["particle", "lattice"], "batch": ["particle", "lattice", "lattice"]}[run]
     assert [kind for kind, _ in launches[run + "1"]] == per_step * {"alone": 6, "batch": 3}[run]
+
+
+@pytest.mark.parametrize("run", ["alone", "batch"])
+def test_lattice_kernels_of_crowded_lattices_wait(launches, run):
+    """400 disks on 124 tiles: the waiting CTAs would crowd on the SMs that the
+    particle kernel leaves free."""
+    assert len(launches[run + "2"]) == len(launches[run + "1"])
+    assert all(early == (kind == "particle") for kind, early in launches[run + "2"])
