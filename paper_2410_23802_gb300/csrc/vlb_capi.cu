@@ -1188,16 +1188,16 @@ static cudaError_t copy_fields(vlb_handle* h, uint32_t mask, double* const (&out
   for (int k = 0; k < 5; ++k)
     if (mask & (1u << k)) field[nfields++] = k;
   std::atomic<int> next{0}, failed{cudaSuccess};
-  auto work = [&]() {
+  auto work = [&](bool helper) {
     std::unique_ptr<float[]> buf;
     if (h->esize == 4) {
       buf.reset(new (std::nothrow) float[(size_t)rows * h->nx]());  // (touched: copies into fresh pages are slow)
-      if (!buf) {
-        failed = cudaErrorMemoryAllocation;
+      if (!buf) {  // (the calling thread takes the pieces that a helper cannot)
+        if (!helper) failed = cudaErrorMemoryAllocation;
         return;
       }
     }
-    cudaError_t e = cudaSetDevice(h->device);
+    cudaError_t e = helper ? cudaSetDevice(h->device) : cudaSuccess;
     for (int q; e == cudaSuccess && failed.load() == cudaSuccess && (q = next.fetch_add(1)) < pieces * nfields;) {
       const int k = field[q / pieces], y0 = q % pieces * rows, n = std::min(rows, h->ny - y0);
       const char* src = static_cast<const char*>(h->macro) + ((size_t)k * h->plane + (size_t)y0 * h->pitch) * h->esize;
@@ -1211,19 +1211,18 @@ static cudaError_t copy_fields(vlb_handle* h, uint32_t mask, double* const (&out
   };
   const size_t most = std::min<size_t>(8, (size_t)nfields * h->nx * h->ny >> 19);
   std::vector<std::thread> others;
-  int device = 0;
-  cudaError_t e = cudaGetDevice(&device);
-  try {
-    others.reserve(8);
-    while (others.size() + 1 < std::min<size_t>(most, std::max(1u, std::thread::hardware_concurrency())))
-      others.emplace_back(work);
-  } catch (const std::exception&) {
-    // no more threads to be had: those that there are do the work
+  if (most > 1) {
+    try {
+      const size_t threads = std::min<size_t>(most, std::max(1u, std::thread::hardware_concurrency()));
+      others.reserve(threads);
+      while (others.size() + 1 < threads) others.emplace_back(work, true);
+    } catch (const std::exception&) {
+      // no more threads to be had: those that there are do the work
+    }
   }
-  work();
+  work(false);
   for (auto& t : others) t.join();
-  if (e == cudaSuccess) e = cudaSetDevice(device);  // (the calling thread's)
-  return failed.load() != cudaSuccess ? static_cast<cudaError_t>(failed.load()) : e;
+  return static_cast<cudaError_t>(failed.load());
 }
 
 extern "C" {

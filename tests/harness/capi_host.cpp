@@ -8,6 +8,8 @@
 //   full        the same with no device memory left, fields read in between, at
 //               step 0 and later: no device allocation, the populations of the
 //               level unchanged
+//   helpers     reads a field with helper threads that get no buffer: the calling
+//               thread takes their pieces
 //   footprint   device bytes of a handle with ellipses and one without, after
 //               the first step: what vlb_device_bytes says
 // Prints "ok", or what differs and exits with 1.
@@ -15,11 +17,22 @@
 #include <cstdlib>
 #include <cstring>
 #include <map>
+#include <new>
+#include <thread>
 #include <string>
 #include <vector>
 
 #include "../../include/vlb.h"
 #include "fake_cuda.h"
+
+// (no-throw array allocations of other threads fail on request)
+static bool g_fail_helpers = false;
+static const std::thread::id g_main = std::this_thread::get_id();
+void* operator new[](size_t n, const std::nothrow_t&) noexcept {
+  return g_fail_helpers && std::this_thread::get_id() != g_main ? nullptr : std::malloc(n);
+}
+void operator delete[](void* p) noexcept { std::free(p); }
+void operator delete[](void* p, size_t) noexcept { std::free(p); }
 
 static int bad(const char* what, int precision) {
   std::printf("%s (precision %d)\n", what, precision);
@@ -106,6 +119,26 @@ static int full() {
   }
   return 0;
 }
+static int helpers() {
+  vlb_params p;
+  vlb_params_default(&p);
+  p.nx = p.ny = 1500;
+  p.precision = VLB_FP32;
+  p.max_particles = 0;
+  vlb_handle* h = nullptr;
+  if (vlb_create(&p, &h) != VLB_OK || vlb_step(h, 0) != VLB_OK) return bad("setup", p.precision);
+  std::vector<double> ux(1500 * 1500, 1.0), T(1500 * 1500, 1.0);
+  g_fail_helpers = true;
+  const vlb_status s = vlb_get_fields(h, VLB_FIELD_UX | VLB_FIELD_T, nullptr, ux.data(), nullptr, T.data(), nullptr);
+  g_fail_helpers = false;
+  if (s != VLB_OK) return bad(vlb_last_error(h), p.precision);
+  float a5;  // (device memory as the stand-in hands it out)
+  std::memset(&a5, 0xA5, sizeof(a5));
+  for (size_t c = 0; c < T.size(); ++c)
+    if (ux[c] != a5 || T[c] != a5) return bad("values missing", p.precision);
+  vlb_destroy(h);
+  return 0;
+}
 static int footprint() {
   for (int precision : {VLB_FP64, VLB_FP32, VLB_FP16_STORE, VLB_BF16_STORE}) {
     for (bool disks : {true, false}) {
@@ -122,7 +155,7 @@ static int footprint() {
 }
 
 int main(int argc, char** argv) {
-  const std::map<std::string, int (*)()> checks = {{"roundtrip", roundtrip}, {"full", full}, {"footprint", footprint}};
+  const std::map<std::string, int (*)()> checks = {{"roundtrip", roundtrip}, {"full", full}, {"helpers", helpers}, {"footprint", footprint}};
   const auto it = argc > 1 ? checks.find(argv[1]) : checks.end();
   if (it == checks.end() || it->second() != 0) return 1;
   std::printf("ok\n");

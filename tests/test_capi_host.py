@@ -28,3 +28,7 @@ def test_device_bytes_counts_every_allocation(harness):
 
 def test_images_allocate_nothing_on_the_device(harness):
     _check(harness, "full")
+
+
+def test_fields_are_read_when_helper_threads_get_no_buffer(harness):
+    _check(harness, "helpers")
