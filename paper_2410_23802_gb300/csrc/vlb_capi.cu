@@ -25,6 +25,8 @@
 #include <utility>
 #include <vector>
 
+#include <unistd.h>
+
 #include "../../include/vlb.h"
 #include "vlb_common.cuh"
 #include "vlb_internal.h"
@@ -1491,35 +1493,45 @@ uint64_t state_bytes(const StateHeader& H) {
 
 }  // extern "C"
 
-// Population buffer b to (out) or from (in) an image's eighteen planes, a
-// direction at a time, split or joined on the device.  The two planes of scratch
-// that takes are the macroscopic planes, which the next read-back computes again:
-// an image allocates nothing.  Those of the initial state cannot be computed
-// again; there the other population buffer serves, which no step has written
-// (its part of the image is zero).  Everything goes through the handle's
-// stream: a pageable copy into the device on the legacy stream may still be
-// under way when its call returns, and the handle's stream would not wait for it.
+// Population buffer b to (out) or from (in) an image's eighteen planes, some
+// directions at a time, split or joined on the device in scratch that an image
+// does not have to allocate: the macroscopic planes, which the next read-back
+// computes again (three directions at a time, seven of 16-bit storage).  Those
+// of the initial state cannot be computed again; there the other population
+// buffer serves, which no step has written (its part of the image is zero), and
+// so it does for the first buffer of an image that is loaded: all directions at
+// once.  Everything goes through the handle's stream: a pageable copy into the
+// device on the legacy stream may still be under way when its call returns, and
+// the handle's stream would not wait for it.
 static cudaError_t copy_populations(vlb_handle* h, int b, char* out, const char* in) {
   const size_t plane = (size_t)h->plane * h->ssize;
-  char* scratch = static_cast<char*>(h->macro);
-  if (out && h->step == 0 && h->macros_valid) {
-    if (b != h->cur) {
-      std::memset(out, 0, 18 * plane);
-      return cudaSuccess;
-    }
-    scratch = static_cast<char*>(h->pop[1 - b]);
-  } else {
-    h->macros_valid = false;
+  const bool initial = out && h->step == 0 && h->macros_valid;
+  if (initial && b != h->cur) {
+    std::memset(out, 0, 18 * plane);
+    return cudaSuccess;
   }
+  const bool other = initial || (in && b == 0);
+  if (!initial) h->macros_valid = false;
+  char* scratch = static_cast<char*>(other ? h->pop[1 - b] : h->macro);
+  const int most = other ? 9 : (int)(7 * h->esize / (2 * h->ssize));
+  // the planes of f, then those of g: one copy of two rows where the rows lie near
+  // (64^2: an image in 175 instead of 227 us), else two copies (a row's pitch has to
+  // stay below 2 GB)
+  auto move = [&](char* to, size_t to_pitch, const char* from, size_t from_pitch, size_t bytes, cudaMemcpyKind kind) {
+    if (9 * plane <= (size_t)1 << 27)
+      return cudaMemcpy2DAsync(to, to_pitch, from, from_pitch, bytes, 2, kind, h->stream);
+    const cudaError_t ef = cudaMemcpyAsync(to, from, bytes, kind, h->stream);
+    return ef != cudaSuccess ? ef : cudaMemcpyAsync(to + to_pitch, from + from_pitch, bytes, kind, h->stream);
+  };
   cudaError_t e = cudaSuccess;
-  for (int i = 0; i < 9 && e == cudaSuccess; ++i) {
-    char* pairs = static_cast<char*>(h->pop[b]) + 2 * plane * i;
-    for (int q = 0; q < 2 && in && e == cudaSuccess; ++q)
-      e = cudaMemcpyAsync(scratch + q * plane, in + (9 * q + i) * plane, plane, cudaMemcpyHostToDevice, h->stream);
+  for (int i = 0; i < 9 && e == cudaSuccess; i += most) {
+    const int k = std::min(most, 9 - i);
+    const size_t bytes = k * plane;
+    if (in) e = move(scratch, bytes, in + i * plane, 9 * plane, bytes, cudaMemcpyHostToDevice);
     if (e == cudaSuccess)
-      e = launch_split_plane(pairs, scratch, scratch + plane, h->plane, h->ssize, in != nullptr, h->stream);
-    for (int q = 0; q < 2 && out && e == cudaSuccess; ++q)
-      e = cudaMemcpyAsync(out + (9 * q + i) * plane, scratch + q * plane, plane, cudaMemcpyDeviceToHost, h->stream);
+      e = launch_split_plane(static_cast<char*>(h->pop[b]) + 2 * plane * i, scratch, scratch + bytes, k * h->plane,
+                             h->ssize, in != nullptr, h->stream);
+    if (out && e == cudaSuccess) e = move(out + i * plane, 9 * plane, scratch, bytes, bytes, cudaMemcpyDeviceToHost);
   }
   const cudaError_t es = cudaStreamSynchronize(h->stream);
   return e != cudaSuccess ? e : es;
@@ -1544,6 +1556,10 @@ vlb_status vlb_save_state(vlb_handle* h, void* buf, uint64_t bytes) {
   CK(h, cudaStreamSynchronize(h->stream));
   if ((s = device_flags(h)) != VLB_OK) return s;
   char* o = static_cast<char*>(buf);
+  // (touched: copies of some MB into fresh pages are slow, 73 MB in twelve 37 ms
+  // against 3 ms)
+  const size_t page = (size_t)std::max(4096l, sysconf(_SC_PAGESIZE));
+  for (uint64_t at = 0; at < state_bytes(H); at += page) *static_cast<volatile char*>(o + at) = 0;
   std::memcpy(o, &H, sizeof(H));
   o += sizeof(H);
   auto get = [&](const void* src, uint64_t n) -> cudaError_t {
@@ -1591,7 +1607,7 @@ vlb_status vlb_load_state(vlb_handle* h, const void* buf, uint64_t bytes) {
     o += n;
     return e;
   };
-  for (int b = 0; b < 2; ++b) {
+  for (int b = 0; b < 2; ++b) {  // (buffer 0 first: see copy_populations)
     CK(h, copy_populations(h, b, nullptr, o));
     o += I.pop_bytes;
     CK(h, put(h->spl[b], I.s_bytes));

@@ -165,7 +165,7 @@ cudaError_t launch_ellipse_batch(const BatchParticles* cases, const BatchEllipse
 cudaError_t launch_audit_f32(const LatticeConst<float>& K, const void* pop, const void* macro,
                              double* scratch, int nblocks, double* out, unsigned* err, cudaStream_t st,
                              int storage);
-// Plane i of (f, g) pairs (n pairs of populations of `bytes` bytes) into the
+// Planes of (f, g) pairs (n pairs of populations of `bytes` bytes) into the
 // planes f, g, or with join from them.
 cudaError_t launch_split_plane(void* pairs, void* f, void* g, long long n, size_t bytes, bool join, cudaStream_t st);
 cudaError_t launch_audit_f64(const LatticeConst<double>& K, const void* pop, const void* macro,
