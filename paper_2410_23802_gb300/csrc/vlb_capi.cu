@@ -203,10 +203,9 @@ static void fill_const(vlb_handle* h, LatticeConst<C>& K) {
   K.cv_f = C(cvf); K.cv_s = C(cvs); K.cref = C(cref); K.lam_f = C(nu / p.prandtl);
   K.rates_mode = C(p.thermal_rates_mode);
   K.bx = C(-p.beta * p.gravity[0]); K.by = C(-p.beta * p.gravity[1]);
-  K.T_ref = C(p.T_ref); K.T_fluid = C(p.T_fluid_init);
+  K.T_fluid = C(p.T_fluid_init);
   K.dT_ref = C(p.T_fluid_init - p.T_ref);
   const double tgf = 0.5 + 3.0 * (nu / p.prandtl) / cref;
-  K.tau_gf = C(tgf);
   K.sj_f = C(1.0 / tgf);
   K.se_f = C(p.thermal_rates_mode == 0 ? 1.0 / (0.5 + 0.25 / (tgf - 0.5)) : 1.0);
   K.k3_cref = C(3.0 / cref);

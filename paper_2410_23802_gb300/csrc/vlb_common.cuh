@@ -28,8 +28,8 @@ __host__ __device__ constexpr C wgt(int i) {
   return i == 0 ? C(4) / C(9) : (i <= 4 ? C(1) / C(9) : C(1) / C(36));
 }
 
-// Tiles of the lattice kernel: one CTA of 32 x TILE_Y threads per 32 x TILE_Y
-// cells (one warp per row of the tile).  TILE_Y is a build-time choice.
+// Tiles of the lattice kernel: 32 x TILE_Y cells, TILE_Y warps (which cells a
+// warp takes depends on the storage: WarpShape).  TILE_Y is a build-time choice.
 #ifndef VLB_TILE_Y
 #define VLB_TILE_Y 4
 #endif
@@ -155,10 +155,6 @@ __device__ __forceinline__ void mes_add(unsigned long long* w, double v, unsigne
   }
   if (hi != 0) atomicAdd(w, (unsigned long long)hi);
 }
-// The total of one accumulator pair as a double.
-__host__ __device__ __forceinline__ double mes_value(unsigned long long hi, unsigned long long lo) {
-  return (double)(long long)hi / MES_SCALE_HI + (double)lo / (MES_SCALE_HI * MES_SCALE_LO);
-}
 
 // Problem constants in the arithmetic type C of the lattice kernel.
 template <class C>
@@ -182,9 +178,9 @@ struct LatticeConst {
   C s_e, s_eps, s_q, s_p;  // the rates themselves (lattices with held particles)
   // thermal (Eqs. 11, 18-22)
   C cv_f, cv_s, cref, lam_f, rates_mode;
-  C bx, by, T_ref, T_fluid;  // buoyancy b = -rho_f beta g; T_f = initial fluid temperature
-  C dT_ref;                  // T_f - T_ref
-  C tau_gf, sj_f, se_f, gk_f;  // thermal rates of a fluid cell (Eqs. 18, 22, 23)
+  C bx, by, T_fluid;       // buoyancy b = -rho_f beta g; T_f = initial fluid temperature
+  C dT_ref;                // T_f - T_ref
+  C sj_f, se_f, gk_f;      // thermal rates of a fluid cell (Eqs. 18, 22, 23)
   C wall_dT[4];              // T_w - T_f per side
   C k3_cref;                 // 3 / c_ref
 };

@@ -172,9 +172,9 @@ __device__ __forceinline__ void held_cell_body(const LatticeConst<float>& K, con
   const C cv = fma_rn(C(1) - fs, K.cv_f, mul_rn(fs, K.cv_s));
   // tau_g from Eq. 22 with alpha_1 = -2; the thermal rates of Eq. 18 (fluid
   // cells use the precomputed values)
-  C tau_g = K.tau_gf, sj = K.sj_f, se = K.se_f, gk = K.gk_f;
+  C sj = K.sj_f, se = K.se_f, gk = K.gk_f;
   if (nown > 0) {
-    tau_g = C(0.5) + lam * K.k3_cref;  // 3 / c_ref
+    const C tau_g = C(0.5) + lam * K.k3_cref;  // 3 / c_ref
     sj = C(1) / tau_g;
     se = (K.rates_mode == C(0)) ? (tau_g - C(0.5)) / (C(0.5) * (tau_g - C(0.5)) + C(0.25)) : C(1);
     gk = -sj * K.k3_cref;  // Eq. 23: -6/(4 + alpha_1) / (c_ref tau_g)

@@ -26,19 +26,19 @@
 
 namespace vlb {
 
-// Tiles covered by [X - R - m, X + R + m] (clipped to the domain), in FP32: the
-// margin m >= 2 cells absorbs the rounding, and the range is computed once per
-// step and stored, so every use of it agrees.
-__device__ __forceinline__ int4 tile_range(const ParticleConst& c, double Xd, double Yd, double Rd) {
-  const float X = float(Xd), Y = float(Yd), e = float(Rd) + float(c.margin);
-  int cx0 = (int)floorf(X - e), cx1 = (int)floorf(X + e);
-  int cy0 = (int)floorf(Y - e), cy1 = (int)floorf(Y + e);
-  cx0 = max(cx0, 0); cy0 = max(cy0, 0);
-  cx1 = min(cx1, c.nx - 1); cy1 = min(cy1, c.ny - 1);
-  if (cx1 < cx0 || cy1 < cy0) return make_int4(0, 0, 0, 0);
-  const int tx0 = cx0 / TILE_X, tx1 = cx1 / TILE_X;
-  const int ty0 = cy0 / TILE_Y, ty1 = cy1 / TILE_Y;
-  return make_int4(tx0, ty0, tx1 - tx0 + 1, ty1 - ty0 + 1);
+// First tile and number of tiles (of T cells) covered along an axis of n cells by
+// [X - R - m, X + R + m], none outside the domain; in FP32: the margin m >= 2
+// cells absorbs the rounding, and the range is computed once per step and
+// stored, so every use of it agrees.
+__device__ __forceinline__ int2 tile_span(const ParticleConst& c, double X, double R, int n, int T) {
+  const float Xf = float(X), e = add_rn(float(R), float(c.margin));
+  const int c0 = max((int)floorf(add_rn(Xf, -e)), 0), c1 = min((int)floorf(add_rn(Xf, e)), n - 1);
+  return c1 < c0 ? make_int2(0, 0) : make_int2(c0 / T, c1 / T - c0 / T + 1);
+}
+// The tiles of a particle along both axes (tx0, ty0, ntx, nty).
+__device__ __forceinline__ int4 tile_range(const ParticleConst& c, double X, double Y, double R) {
+  const int2 x = tile_span(c, X, R, c.nx, TILE_X), y = tile_span(c, Y, R, c.ny, TILE_Y);
+  return x.y == 0 || y.y == 0 ? make_int4(0, 0, 0, 0) : make_int4(x.x, y.x, x.y, y.y);
 }
 
 // Raster record of particle p at centre (X, Y) with velocity (ux, uy, om);
@@ -126,15 +126,9 @@ __device__ __forceinline__ UpdateLane update_position(const ParticleConst& c, co
     const double f = __dadd_rn(X, -double(u.cell));
     u.fh = float(f);
     u.fl = float(__dadd_rn(f, -double(u.fh)));
-    // tiles covered along this axis by [X - R - m, X + R + m], in FP32: the
-    // margin m >= 2 cells absorbs the rounding
-    const float Xf = float(X), e = add_rn(float(u.R), float(c.margin));
-    const int c0 = max((int)floorf(add_rn(Xf, -e)), 0), c1 = min((int)floorf(add_rn(Xf, e)), n - 1);
-    const int T = k == 0 ? TILE_X : TILE_Y;
-    if (c1 >= c0) {
-      u.t0 = c0 / T;
-      u.nt = c1 / T - u.t0 + 1;
-    }
+    const int2 span = tile_span(c, X, u.R, n, k == 0 ? TILE_X : TILE_Y);
+    u.t0 = span.x;
+    u.nt = span.y;
   }
   // outside along one axis: no tiles at all
   const int other = __shfl_xor_sync(0xffffffffu, u.nt, 1);
@@ -161,7 +155,7 @@ __device__ __forceinline__ void update_velocity(const ParticleConst& c, const Pa
   const int k = u.k;
   const double* kp = P.pk + 8 * (long long)p;  // 1/M, 1/I, M_in, I_in, body factor, wall factor
   const double inv_m = kp[k == 2 ? 1 : 0], m_in = kp[k == 2 ? 3 : 2], body = kp[4], wall = kp[5];
-  // the total force or torque of the accumulators (mes_value)
+  // the total force or torque: word 0 in units of 2^-40, word 1 of 2^-104
   const double Fm = __fma_rn((double)(long long)u.acc0, 1.0 / MES_SCALE_HI,
                              __dmul_rn((double)u.acc1, 1.0 / (MES_SCALE_HI * MES_SCALE_LO)));
   // wall contact forces: walls x-, x+ (lane 0), y-, y+ (lane 1), none on open
