@@ -14,12 +14,12 @@ namespace vlb {
 //
 // What bounds it (GB300, one launch per step, FP32 at 152 B per cell update):
 //   FP32, 2048^2 with 2048 disks: memory and the particle tiles' chain of list,
-//     record and band table; 110.3 us = 5.78 TB/s (127 us before: a list per
+//     record and band table; 111.0 us = 5.75 TB/s (127 us before: a list per
 //     CTA behind a barrier, exchange sums over shared memory, f and g in planes
 //     of their own, both collisions by the full moment matrices).  Without
 //     particles 96 us = 6.6 TB/s.
-//   16-bit storage, same case: instruction issue, 527 per warp of 32 cells
-//     (880 before); FP16 92 us, BF16 91 us.
+//   16-bit storage, same case: instruction issue, 539 per warp of 32 cells
+//     (880 before); FP16 92.6 us, BF16 92.7 us.
 //   FP64, 100 x 400: the FP64 pipe (67 % busy); 37 us (56 before).
 //   A lattice of less than a wave of warps (100 x 400 FP32): the latency of one
 //     cell, 3.7 us.
@@ -194,8 +194,8 @@ cudaError_t launch_audit_f64(const LatticeConst<double>& K, const void* pop, con
   return audit<double, double>(K, pop, macro, scratch, nblocks, out, err, st);
 }
 
-// One plane of (f_i, g_i) pairs to or from its two planes f_i, g_i (the form
-// of a state image); W: an unsigned word of a population's size.
+// Planes of (f_i, g_i) pairs to or from as many planes f_i and g_i (the form of a
+// state image), n pairs in all; W: an unsigned word of a population's size.
 template <class W>
 __global__ void split_plane_kernel(W* __restrict__ pairs, W* __restrict__ f, W* __restrict__ g, long long n, int join) {
   for (long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x; c < n; c += (long long)gridDim.x * blockDim.x) {
